@@ -11,6 +11,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "flow.cuh"
 #include "solve.cuh"
 
 using namespace spt;
@@ -135,6 +136,10 @@ struct sptrsv_plan_st {
     // direction, the first level of the thin run holding every level
     int32_t thin_rows = 0, seg_rows = -1;
     int32_t *d_seg[2] = {nullptr, nullptr};
+    // cluster flow schedule of each direction ([0] forward, [1] transpose),
+    // built when the hybrid mode is chosen; off: could not be built
+    FlowSched flow[2];
+    bool flow_ready[2] = {false, false}, flow_off = false;
     // row-major copies of a column-major right-hand-side block and its
     // solution (sptrsv_solve_layout), grown on demand
     void *d_lay = nullptr;
@@ -479,6 +484,112 @@ sptrsv_status ensure_hybrid(sptrsv_plan p)
     return SPTRSV_OK;
 }
 
+// Tables of the cluster flow schedule (flow.cuh) of one direction.  One block
+// of the cluster per 24 rows of the mean level: below that another block does
+// not shorten a level (power-law DAG, 63 rows a level: 2 blocks 10.4 ms, 4
+// 9.6 ms, 16 9.2 ms transpose).  Beyond 8 blocks only for very wide levels:
+// with 16 the 2D Laplacian (512 rows a level) gains 6 % at one right-hand
+// side, but the GPU holds too few such clusters for eight (5.0 against 3.5 ms).
+sptrsv_status build_flow(sptrsv_plan p, int dir)
+{
+    const PlanMat &M = p->M;
+    const int32_t n = M.L.n, L = M.nlevels;
+    const size_t nn = (size_t)n, nc = (size_t)L * kFlowClasses;
+    cudaStream_t s = p->h->stream;
+    const bool f64 = p->dtype == SPTRSV_F64;
+    if (n > kFlowMaxRows) return SPTRSV_ENOTSUP;
+    int csize = 1;
+    const double width = (double)n / L;
+    while (csize < (width >= 768.0 ? kFlowMaxCluster : 8) && width > 24.0 * csize) csize <<= 1;
+    while (csize > 1 && !flow_cluster_fits(csize, f64)) csize >>= 1;
+    if (!flow_cluster_fits(csize, f64)) return SPTRSV_ENOTSUP;
+    const int32_t *ptr = dir ? M.d_cp : M.L.row_ptr, *idx = dir ? M.d_crow : M.L.col_idx;
+    int32_t *order = nullptr;
+    cudaError_t e = cudaMallocAsync(&order, sizeof(int32_t) * (4 * nn + nc), s);
+    if (e != cudaSuccess) return from_cuda(e);
+    int32_t *iperm = order + nn, *counts = iperm + 3 * nn;
+    uint32_t *meta = reinterpret_cast<uint32_t *>(iperm + nn), *mask = meta + nn;
+    e = flow_order(ptr, M.d_lev, n, L, dir != 0, order, iperm, counts, s);
+    std::vector<int32_t> cnt(nc);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(cnt.data(), counts, sizeof(int32_t) * nc, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    // groups of one level and class, an equal share of every level's groups,
+    // in order, to each block of the cluster
+    std::vector<std::vector<FlowGroup>> by((size_t)csize);
+    std::vector<FlowGroup> lev;
+    int32_t q = 0;
+    static const int llpr[kFlowClasses] = {0, 2, 4, 5};
+    for (int32_t l = 0; l < L && e == cudaSuccess; ++l) {
+        lev.clear();
+        for (int c = 0; c < kFlowClasses; ++c) {
+            int32_t left = cnt[(size_t)l * kFlowClasses + c];
+            for (const int32_t most = 32 >> llpr[c]; left > 0;) {
+                const int32_t take = std::min(most, left);
+                lev.push_back(FlowGroup{q, take, llpr[c]});
+                q += take;
+                left -= take;
+            }
+        }
+        const int64_t G = (int64_t)lev.size();
+        for (int64_t g = 0; g < G; ++g) by[(size_t)(g * csize / G)].push_back(lev[(size_t)g]);
+    }
+    std::vector<FlowGroup> all;
+    std::vector<int32_t> gptr(1, 0);
+    for (const auto &v : by) {
+        all.insert(all.end(), v.begin(), v.end());
+        gptr.push_back((int32_t)all.size());
+    }
+    const size_t ns = 32 * std::max<size_t>(all.size(), 1), w = f64 ? 8 : 4;
+    FlowLane *lanes = nullptr;
+    uint4 *codes = nullptr;
+    int2 *src = nullptr;
+    uint32_t *ecode = nullptr;
+    FlowGroup *groups = nullptr;
+    int32_t *d_gptr = nullptr;
+    FlowSched F{};
+    if (e == cudaSuccess) e = p->alloc(&lanes, sizeof(FlowLane) * ns);
+    if (e == cudaSuccess) e = p->alloc(&codes, sizeof(uint4) * ns);
+    if (e == cudaSuccess) e = p->alloc(&src, sizeof(int2) * ns);
+    if (e == cudaSuccess) e = p->alloc(&ecode, sizeof(uint32_t) * (size_t)M.L.nnz);
+    if (e == cudaSuccess) e = p->alloc(&F.vals, 4 * w * ns);
+    if (e == cudaSuccess) e = p->alloc(&F.inv, w * ns);
+    if (e == cudaSuccess) e = p->alloc(&d_gptr, sizeof(int32_t) * gptr.size());
+    if (e == cudaSuccess) e = cudaMallocAsync(&groups, sizeof(FlowGroup) * std::max<size_t>(all.size(), 1), s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(groups, all.data(), sizeof(FlowGroup) * all.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(d_gptr, gptr.data(), sizeof(int32_t) * gptr.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess)
+        e = flow_tables(ptr, idx, n, dir != 0, f64, order, iperm, groups, d_gptr, (int32_t)all.size(), csize, meta,
+                        mask, lanes, codes, src, ecode, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaFreeAsync(order, s);
+    if (groups) cudaFreeAsync(groups, s);
+    if (e != cudaSuccess) return from_cuda(e);
+    F.lanes = lanes;
+    F.codes = codes;
+    F.src = src;
+    F.ecode = ecode;
+    F.gptr = d_gptr;
+    F.n = n;
+    F.csize = csize;
+    F.ngroups = (int32_t)all.size();
+    p->flow[dir] = F;
+    p->flow_ready[dir] = true;
+    return SPTRSV_OK;
+}
+
+// Whether solves of direction dir run the cluster flow schedule: the hybrid
+// mode with its automatic threshold (one synchronisation-free run in level
+// order) and grid.  Where the tables cannot be had, the grid-wide hybrid
+// kernel runs.
+bool use_flow(sptrsv_plan p, int dir)
+{
+    if (p->mode != SPTRSV_MODE_HYBRID || p->thin_rows != 0 || p->flow_off || p->M.L.n == 0) return false;
+    if (p->grid_level != p->grid_level_max) return false;
+    if (p->flow_ready[dir]) return true;
+    if (build_flow(p, dir) != SPTRSV_OK) p->flow_off = true;
+    return !p->flow_off;
+}
+
 // Mode from the mean level width: narrow (deep) systems stay on one SM,
 // very wide levels go level by level (row-order sync-free solving keeps
 // only the rows in flight near the wavefront and idles on wide, far-reaching
@@ -531,6 +642,10 @@ sptrsv_status solve_impl(sptrsv_plan p, const void *b, void *x, int32_t nrhs, in
         break;
     }
     case SPTRSV_MODE_HYBRID: {
+        if (use_flow(p, trans ? 1 : 0)) {
+            e = solve_flow<T>(A, p->flow[trans ? 1 : 0], R, trans, p->withhold, sy.w, s);
+            break;
+        }
         sptrsv_status st = ensure_chunks(p);
         if (st == SPTRSV_OK) st = ensure_hybrid(p);
         if (st != SPTRSV_OK) return st;
@@ -712,6 +827,8 @@ extern "C" sptrsv_status sptrsv_plan_create(sptrsv_handle h, const sptrsv_csr *L
     st = ensure_chunks(p);
     if (st == SPTRSV_OK) st = from_cuda(cudaStreamSynchronize(h->stream));
     if (st != SPTRSV_OK) { sptrsv_plan_destroy(p); return st; }
+    use_flow(p, 0);
+    if (p->have_csc) use_flow(p, 1);
     *plan = p;
     return SPTRSV_OK;
 }
@@ -780,6 +897,8 @@ extern "C" sptrsv_status sptrsv_plan_set(sptrsv_plan p, int32_t mode, int32_t ro
     if (rhs_tile) p->kt = rhs_tile;
     sptrsv_status st = ensure_chunks(p);
     if (st != SPTRSV_OK) return st;
+    use_flow(p, 0);
+    if (p->have_csc) use_flow(p, 1);
     return from_cuda(cudaStreamSynchronize(p->h->stream));
 }
 
