@@ -107,8 +107,9 @@ typedef struct {
     int32_t rows_per_warp;   /* 1,2,4,8,16,32 (lanes per row = 32/rows_per_warp); 0 = auto */
     int32_t rhs_tile;        /* right-hand sides per pass: 1,2,4,8,16; 0 = auto.
                                 Block mode and batched plans: columns per
-                                thread block (1,2,4,8); wider right-hand
-                                sides run as independent column tiles      */
+                                thread block (1,2,4,8; at most 4 with 32
+                                rows per warp); wider right-hand sides run
+                                as independent column tiles                */
     int32_t build_transpose; /* non-zero: prepare sptrsv_solve_transpose / grad  */
     int64_t wait_limit_us;   /* longest a device wait may take before the solve
                                 gives up with SPTRSV_ETIMEOUT (microseconds);
@@ -240,9 +241,9 @@ sptrsv_status sptrsv_plan_set(sptrsv_plan plan, int32_t mode, int32_t rows_per_w
 sptrsv_status sptrsv_solve(sptrsv_plan plan, const void *b, void *x, int32_t nrhs, int64_t ld);
 
 /* Adjoint of the solve: g_b = L^{-T} g_x, processed in reverse level /
- * reverse row order.  Requires build_transpose.  Asynchronous.  First
- * gathers L's current values into CSC order (one elementwise launch, plan-
- * owned buffer), so values may change between calls.                      */
+ * reverse row order.  Requires build_transpose.  Asynchronous.  L's current
+ * values are read on every call (most schedules first gather them into CSC
+ * order in a plan-owned buffer), so values may change between calls.      */
 sptrsv_status sptrsv_solve_transpose(sptrsv_plan plan, const void *gx, void *gb, int32_t nrhs,
                                      int64_t ld);
 
@@ -339,9 +340,9 @@ sptrsv_status sptrsv_batch_plan_set_direction(sptrsv_plan plan, int32_t directio
 #define SPTRSV_BATCH_LEVEL 2
 sptrsv_status sptrsv_batch_plan_set_schedule(sptrsv_plan plan, int32_t direction,
                                              const int32_t *schedule);
-/* All systems in one persistent launch (plus a tiny reset launch; the
- * transpose solve also gathers the values into CSC order first): no host
- * work per matrix, so the call can be captured in a CUDA graph.            */
+/* All systems in one persistent launch (plus a tiny reset launch and one
+ * that lays the current values out for it): no host work per matrix, so the
+ * call can be captured in a CUDA graph.                                    */
 sptrsv_status sptrsv_batch_solve(sptrsv_plan plan, const void *b, void *x);
 sptrsv_status sptrsv_batch_solve_transpose(sptrsv_plan plan, const void *gx, void *gb);
 sptrsv_status sptrsv_batch_grad_vals(sptrsv_plan plan, const void *gb, const void *x,

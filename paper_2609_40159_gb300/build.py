@@ -17,7 +17,7 @@ LIB = os.path.join(HERE, "libsptrsv_gb300.so")
 # bounds-checked debug variant: every gather index checked (SPTRSV_CHECKED)
 BUILD_CHECKED = os.path.join(HERE, "_build_checked")
 LIB_CHECKED = os.path.join(HERE, "libsptrsv_gb300_checked.so")
-SOURCES = ["api.cu", "analyze.cu", "prims.cu", "rewrite.cu", "solve.cu", "flow.cu", "batch.cu", "noalloc.cu"]
+SOURCES = ["api.cu", "analyze.cu", "prims.cu", "rewrite.cu", "solve.cu", "flow.cu", "strip.cu", "batch.cu", "noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
 

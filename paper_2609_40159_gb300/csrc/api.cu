@@ -13,6 +13,7 @@
 
 #include "flow.cuh"
 #include "solve.cuh"
+#include "strip.cuh"
 
 using namespace spt;
 
@@ -68,6 +69,14 @@ int default_rpw(int32_t n, int64_t nnz, int64_t long_rows = 0)
     return 1;
 }
 
+// The same for block-local solves, which stage up to 16 dependencies a row on
+// the previous group and 16 older ones: one lane per row for longer rows too.
+int block_rpw(int32_t n, int64_t nnz, int64_t long_rows = 0)
+{
+    const int r = default_rpw(n, nnz, long_rows);
+    return r == 16 && (double)nnz / n <= 20.0 ? 32 : r;
+}
+
 int default_kt(int k)
 {
     int kt = 1;
@@ -109,6 +118,8 @@ struct PlanMat {
     int32_t *d_iperm = nullptr;
     LevelGroup *d_lgroups[2] = {nullptr, nullptr};
     int32_t n_lgroups[2] = {0, 0};
+    // strips of each direction (block-local in-order solves)
+    Strips strips[2]{};
 };
 
 struct sptrsv_plan_st {
@@ -154,6 +165,7 @@ struct sptrsv_plan_st {
     // column tile, geometry), their launch order, shared memory and grid
     struct Geom {
         std::vector<int32_t> rpw, tile, sched;
+        bool csc_vals = false;  // some item reads L's values in CSC order
         BatchItem *d_items = nullptr;
         int32_t *d_order = nullptr;
         int32_t nitems = 0;
@@ -484,6 +496,62 @@ sptrsv_status ensure_hybrid(sptrsv_plan p)
     return SPTRSV_OK;
 }
 
+// Strips (strip.cuh) of one direction of systems that have none; left out when
+// their memory cannot be had (then the solves take several lanes per row).
+void build_strips(sptrsv_plan p, const std::vector<PlanMat *> &mats, int dir)
+{
+    if (mats.empty()) return;
+    const size_t nm = mats.size();
+    std::vector<StripSrc> src(nm);
+    int64_t ng = 0, nnz = 0;
+    for (size_t m = 0; m < nm; ++m) {
+        const PlanMat &M = *mats[m];
+        src[m] = StripSrc{dir ? M.d_cp : M.L.row_ptr, dir ? M.d_crow : M.L.col_idx, ng, nnz, M.L.n};
+        ng += ((int64_t)M.L.n + 31) / 32;
+        nnz += M.L.nnz;
+    }
+    cudaStream_t s = p->h->stream;
+    char *tmp = nullptr, *tab = nullptr;
+    const size_t b_src = sizeof(StripSrc) * nm, b_ofs = 4 * ((size_t)ng + 1);
+    cudaError_t e = cudaMallocAsync(&tmp, 8 + b_src + 4 * nm + 8 * (size_t)ng + b_ofs, s);
+    if (e != cudaSuccess) { cudaGetLastError(); return; }
+    StripBuild B{};
+    B.total = reinterpret_cast<int64_t *>(tmp);
+    B.src = reinterpret_cast<StripSrc *>(tmp + 8);
+    B.far = reinterpret_cast<int32_t *>(tmp + 8 + b_src);
+    B.units = B.far + nm;
+    B.bits = reinterpret_cast<uint32_t *>(B.units + ng);
+    B.ofs = B.bits + ng;
+    B.nsrc = (int32_t)nm;
+    B.ng = ng;
+    B.trans = dir != 0;
+    B.f64 = p->dtype == SPTRSV_F64;
+    B.ring_most = strip_ring_most(B.f64, p->batched);
+    std::vector<int32_t> far(nm);
+    int64_t total = 0;
+    e = cudaMemcpyAsync(tmp + 8, src.data(), b_src, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(B.far, 0, 4 * nm, s);
+    if (e == cudaSuccess) e = strip_sizes(B, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&total, B.total, sizeof(total), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(far.data(), B.far, 4 * nm, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess && total > INT32_MAX) e = cudaErrorMemoryAllocation;  // (32 GB)
+    const size_t b_blocks = 16 * (size_t)total;
+    if (e == cudaSuccess) e = p->alloc(&tab, b_blocks + b_ofs + 2 * (size_t)nnz);
+    if (e == cudaSuccess) {
+        uint32_t *ofs = reinterpret_cast<uint32_t *>(tab + b_blocks);
+        uint16_t *ecode = reinterpret_cast<uint16_t *>(tab + b_blocks + b_ofs);
+        e = cudaMemcpyAsync(ofs, B.ofs, b_ofs, cudaMemcpyDeviceToDevice, s);
+        if (e == cudaSuccess) e = strip_tables(B, ofs, reinterpret_cast<unsigned char *>(tab), ecode, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        for (size_t m = 0; m < nm && e == cudaSuccess; ++m)
+            mats[m]->strips[dir] = Strips{reinterpret_cast<unsigned char *>(tab), ofs + src[m].g0, ecode + src[m].e0,
+                                          strip_ring(far[m], B.ring_most)};
+    }
+    cudaFreeAsync(tmp, s);
+    if (e != cudaSuccess) cudaGetLastError();
+}
+
 // Tables of the cluster flow schedule (flow.cuh) of one direction.  One block
 // of the cluster per 24 rows of the mean level: below that another block does
 // not shorten a level (power-law DAG, 63 rows a level: 2 blocks 10.4 ms, 4
@@ -590,6 +658,16 @@ bool use_flow(sptrsv_plan p, int dir)
     return !p->flow_off;
 }
 
+// Builds the tables of the plan's mode, so that a solve launches kernels only.
+void prepare_schedules(sptrsv_plan p)
+{
+    for (int dir = 0; dir < (p->have_csc ? 2 : 1); ++dir) {
+        use_flow(p, dir);
+        if (p->mode == SPTRSV_MODE_BLOCK && p->rpw == 32 && p->M.L.n > 0 && !p->M.strips[dir].blocks)
+            build_strips(p, {&p->M}, dir);
+    }
+}
+
 // Mode from the mean level width: narrow (deep) systems stay on one SM,
 // very wide levels go level by level (row-order sync-free solving keeps
 // only the rows in flight near the wavefront and idles on wide, far-reaching
@@ -615,7 +693,13 @@ sptrsv_status solve_impl(sptrsv_plan p, const void *b, void *x, int32_t nrhs, in
     cudaStream_t s = p->h->stream;
     Sys<T> A = sys_of<T>(M, p->h->d_status);
     Rhs<T> R{(const T *)b, (T *)x, ld, nrhs};
-    if (trans) {
+    int mode = p->mode;
+    if (mode == SPTRSV_MODE_BLOCK && !block_mode_supported(nrhs, sizeof(T) == 8)) mode = SPTRSV_MODE_SYNCFREE;
+    const int dir = trans ? 1 : 0;
+    // schedules that lay the values out themselves
+    const bool strips = mode == SPTRSV_MODE_BLOCK && p->rpw == 32 && M.strips[dir].blocks != nullptr;
+    const bool flow = mode == SPTRSV_MODE_HYBRID && use_flow(p, dir);
+    if (trans && !strips && !flow) {
         cudaError_t eg = csc_values<T>(M.d_tmap, (const T *)M.L.vals, (T *)M.d_cv, M.L.nnz, s);
         if (eg != cudaSuccess) return from_cuda(eg);
     }
@@ -625,8 +709,6 @@ sptrsv_status solve_impl(sptrsv_plan p, const void *b, void *x, int32_t nrhs, in
     if (nrhs == 1) sy.vflags = p->d_vflags;
     const int kt = std::min(p->kt, default_kt(nrhs));
     cudaError_t e = cudaSuccess;
-    int mode = p->mode;
-    if (mode == SPTRSV_MODE_BLOCK && !block_mode_supported(nrhs, sizeof(T) == 8)) mode = SPTRSV_MODE_SYNCFREE;
     switch (mode) {
     case SPTRSV_MODE_LEVEL_LAUNCH:
         e = solve_level_launch<T>(A, M.d_perm, M.h_level_ptr, R, trans, s);
@@ -642,8 +724,8 @@ sptrsv_status solve_impl(sptrsv_plan p, const void *b, void *x, int32_t nrhs, in
         break;
     }
     case SPTRSV_MODE_HYBRID: {
-        if (use_flow(p, trans ? 1 : 0)) {
-            e = solve_flow<T>(A, p->flow[trans ? 1 : 0], R, trans, p->withhold, sy.w, s);
+        if (flow) {
+            e = solve_flow<T>(A, p->flow[dir], R, trans, p->withhold, sy.w, s);
             break;
         }
         sptrsv_status st = ensure_chunks(p);
@@ -656,7 +738,8 @@ sptrsv_status solve_impl(sptrsv_plan p, const void *b, void *x, int32_t nrhs, in
     }
     case SPTRSV_MODE_BLOCK: {
         const double width = M.nlevels > 0 ? (double)M.L.n / M.nlevels : 1.0;
-        e = solve_block<T>(A, R, p->rpw, kt, trans, sy, block_warps_for(width, p->rpw), s);
+        const int rpw = p->rpw == 32 && !strips ? 16 : p->rpw;
+        e = solve_block<T>(A, M.strips[dir], R, rpw, trans, sy, block_warps_for(width, rpw), s);
         break;
     }
     default:
@@ -804,7 +887,8 @@ extern "C" sptrsv_status sptrsv_plan_create(sptrsv_handle h, const sptrsv_csr *L
         if (e == cudaSuccess) e = cudaMemcpyAsync(&nlong, d, sizeof(nlong), cudaMemcpyDeviceToHost, h->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
         if (e != cudaSuccess) { sptrsv_plan_destroy(p); return from_cuda(e); }
-        p->rpw = default_rpw(L->n, L->nnz, (int64_t)nlong);
+        p->rpw = p->mode == SPTRSV_MODE_BLOCK ? block_rpw(L->n, L->nnz, (int64_t)nlong)
+                                              : default_rpw(L->n, L->nnz, (int64_t)nlong);
     }
     // the hybrid schedule waits row by row on flags: 4 rows per warp (8
     // lanes a row; on the 2D Laplacian 3.2 ms against 4.2 ms with one row
@@ -827,8 +911,7 @@ extern "C" sptrsv_status sptrsv_plan_create(sptrsv_handle h, const sptrsv_csr *L
     st = ensure_chunks(p);
     if (st == SPTRSV_OK) st = from_cuda(cudaStreamSynchronize(h->stream));
     if (st != SPTRSV_OK) { sptrsv_plan_destroy(p); return st; }
-    use_flow(p, 0);
-    if (p->have_csc) use_flow(p, 1);
+    prepare_schedules(p);
     *plan = p;
     return SPTRSV_OK;
 }
@@ -897,8 +980,7 @@ extern "C" sptrsv_status sptrsv_plan_set(sptrsv_plan p, int32_t mode, int32_t ro
     if (rhs_tile) p->kt = rhs_tile;
     sptrsv_status st = ensure_chunks(p);
     if (st != SPTRSV_OK) return st;
-    use_flow(p, 0);
-    if (p->have_csc) use_flow(p, 1);
+    prepare_schedules(p);
     return from_cuda(cudaStreamSynchronize(p->h->stream));
 }
 
@@ -1033,10 +1115,28 @@ sptrsv_status rebuild_items(sptrsv_plan p, int dir)
     std::vector<BatchItem> items;
     std::vector<double> est;
     size_t smem = 16;
+    G.csc_vals = false;
+    auto takes_strips = [&](int m) { return G.rpw[m] == 32 && G.sched[m] == kSchedInOrder && p->mats[m].L.n > 0; };
+    std::vector<PlanMat *> need;
+    if (dir == 0 || p->have_csc)
+        for (int m = 0; m < nmat; ++m)
+            if (takes_strips(m) && !p->mats[m].strips[dir].blocks) need.push_back(&p->mats[m]);
+    if (!need.empty()) {
+        build_strips(p, need, dir);
+        for (int m = 0; m < nmat; ++m) p->h_mats[m].strips[dir] = p->mats[m].strips[dir];
+        cudaError_t e = cudaStreamSynchronize(p->h->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpy(p->d_mats, p->h_mats.data(), sizeof(BatchMat) * nmat, cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) return from_cuda(e);
+    }
     for (int m = 0; m < nmat; ++m) {
-        const PlanMat &M = p->mats[m];
+        PlanMat &M = p->mats[m];
         const int k = p->h_mats[m].k;
-        const int tile = G.tile[m];
+        int tile = G.tile[m];
+        // one lane per row, over the strips
+        const bool one_lane = G.rpw[m] == 32 && (!takes_strips(m) || M.strips[dir].blocks || (dir == 1 && !p->have_csc));
+        G.csc_vals = G.csc_vals || G.sched[m] == kSchedLevel || !one_lane;
+        if (G.sched[m] == kSchedInOrder && one_lane) tile = std::min(tile, 4);
         for (int r0 = 0; r0 < k; r0 += tile) {
             BatchItem I{};
             I.mat = m;
@@ -1044,13 +1144,18 @@ sptrsv_status rebuild_items(sptrsv_plan p, int dir)
             I.kt = std::min(tile, k - r0);
             I.KT = pow2_at_least(I.kt);
             I.sched = G.sched[m];
-            I.rpw = I.sched == kSchedLevel ? 32 : G.rpw[m];
-            I.nw = I.sched == kSchedLevel
-                       ? kBatchWarps
-                       : std::min(kBatchWarps,
-                                  block_warps_for(M.nlevels > 0 ? (double)M.L.n / M.nlevels : 1.0, I.rpw));
-            block_geometry(I.rpw, I.KT, f64, I.nw, &I.kc, &I.P, kBatchSmemGrow);
-            smem = std::max(smem, block_smem_bytes(I.rpw, I.KT, I.kc, f64, I.nw));
+            I.rpw = I.sched == kSchedLevel ? 32 : G.rpw[m] == 32 && !one_lane ? 16 : G.rpw[m];
+            if (I.sched == kSchedInOrder && I.rpw == 32) {
+                I.nw = kBatchWarps;
+                smem = std::max(smem, strip_smem(M.strips[dir].ring, I.KT, f64, kBatchWarps));
+            } else {
+                I.nw = I.sched == kSchedLevel
+                           ? kBatchWarps
+                           : std::min(kBatchWarps,
+                                      block_warps_for(M.nlevels > 0 ? (double)M.L.n / M.nlevels : 1.0, I.rpw));
+                block_geometry(I.rpw, I.KT, f64, I.nw, &I.kc, &I.P, kBatchSmemGrow);
+                smem = std::max(smem, block_smem_bytes(I.rpw, I.KT, I.kc, f64));
+            }
             items.push_back(I);
             // in order: a chain of n / 32 row groups whose cost grows with
             // the tile width; level-ordered: a chain of one or more groups per
@@ -1210,7 +1315,10 @@ extern "C" sptrsv_status sptrsv_batch_plan_create(sptrsv_handle h, int32_t nmat,
     p->h_mats.resize((size_t)nmat);
     for (int d = 0; d < 2; ++d) {
         p->geo[d].rpw.assign((size_t)nmat, 32);
-        p->geo[d].tile.assign((size_t)nmat, 4);
+        // (two columns an item: on 256 training systems of 1,000-40,000 rows,
+        // FP32, 3.43 / 3.03 / 3.40 ms a step with 1 / 2 / 4; on 32 small FP64
+        // ones 0.41 / 0.42 / 0.63 ms)
+        p->geo[d].tile.assign((size_t)nmat, 2);
         p->geo[d].sched.assign((size_t)nmat, kSchedInOrder);
     }
     int64_t ktot = 0;
@@ -1242,7 +1350,7 @@ extern "C" sptrsv_status sptrsv_batch_plan_create(sptrsv_handle h, int32_t nmat,
         p->vals_off[m + 1] = p->vals_off[m] + M.L.nnz;
         p->row_off[m + 1] = p->row_off[m] + M.L.n;
         for (int d = 0; d < 2; ++d) {
-            p->geo[d].rpw[m] = opts && opts[m].rows_per_warp ? opts[m].rows_per_warp : default_rpw(M.L.n, M.L.nnz);
+            p->geo[d].rpw[m] = opts && opts[m].rows_per_warp ? opts[m].rows_per_warp : block_rpw(M.L.n, M.L.nnz);
             if (opts && opts[m].rhs_tile) p->geo[d].tile[m] = opts[m].rhs_tile;
         }
         ktot += B.k;
@@ -1351,9 +1459,13 @@ sptrsv_status batch_solve_impl(sptrsv_plan p, const void *b, void *x, bool trans
     p->last_dir = trans ? 1 : 0;
     Waiter w{p->h->d_status, &p->d_ctl->abort_flag, p->spin};
     cudaError_t e = cudaSuccess;
-    if (trans)
+    if (trans && G.csc_vals)
         e = p->dtype == SPTRSV_F64 ? batch_csc_values<double>(p->d_mats, p->d_ctiles, p->n_ctiles, p->h->stream)
                                    : batch_csc_values<float>(p->d_mats, p->d_ctiles, p->n_ctiles, p->h->stream);
+    if (e == cudaSuccess)
+        e = p->dtype == SPTRSV_F64
+                ? strip_stage_batch<double>(p->d_mats, p->d_gchunks, p->n_gchunks, trans, p->h->stream)
+                : strip_stage_batch<float>(p->d_mats, p->d_gchunks, p->n_gchunks, trans, p->h->stream);
     if (e != cudaSuccess) return from_cuda(e);
     if (p->dtype == SPTRSV_F64)
         e = batch_solve<double>(p->d_mats, G.d_items, G.nitems, G.d_order, (const double *)b, (double *)x,

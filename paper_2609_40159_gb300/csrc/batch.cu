@@ -2,10 +2,11 @@
 // each with its own number of right-hand sides, in ONE persistent launch.
 // Thread blocks take work items -- one system and a tile of at most 8 of its
 // right-hand-side columns -- from a ticket (longest estimated chain first)
-// and run the block algorithm on them; no host work per system, so a batch
-// solve is two kernel nodes in a CUDA graph.  The adjoint's elementwise
+// and run a block algorithm on them (strip.cuh, block.cuh); no host work per
+// system, so a batch solve is a few kernel nodes in a CUDA graph.  The adjoint's elementwise
 // parts (value gradient, T^T) walk plan-time tables of 32-row chunks.
 #include "block.cuh"
+#include "strip.cuh"
 
 namespace spt {
 
@@ -28,13 +29,9 @@ __device__ __forceinline__ Sys<T> sys_of(const BatchMat &M)
 }
 
 template <class T, int KT, bool TR>
-__device__ __forceinline__ bool run_one(const BatchMat &M, const BatchItem &I, unsigned char *raw,
-                                        const T *b, const T *bt, T *x, const Waiter &w, int withhold)
+__device__ __forceinline__ void run_one(const BatchMat &M, const BatchItem &I, unsigned char *raw,
+                                        const T *b, const T *bt, T *x, int *s_bad, const Waiter &w, int withhold)
 {
-    const int ring = I.kc * I.rpw;
-    BlockSmem<T, KT> sm = carve_block_smem<T, KT>(raw, ring, I.kc, I.nw);
-    reset_block_smem<T, KT>(sm, ring, I.kc);
-    __syncthreads();
     Sys<T> A = sys_of<T>(M);
     A.chk = w.status;
     // a rewritten system's forward right-hand side b + T b was formed by the
@@ -49,13 +46,22 @@ __device__ __forceinline__ bool run_one(const BatchMat &M, const BatchItem &I, u
     // test hook: a withheld row (counted over all systems) is never published
     const int64_t wh = (int64_t)withhold - M.row_off;
     const int local = (withhold >= 0 && wh >= 0 && wh < M.n) ? (int)wh : -1;
-    const bool ok = I.sched == kSchedLevel
-                        ? block_solve_levels<T, KT, TR>(A, R, M.perm, M.iperm, M.lgroups[TR ? 1 : 0],
-                                                        M.nlgroups[TR ? 1 : 0], I.kc, I.nw, sm, w, local)
-                        : block_solve_any<T, KT, TR, false>(A, R, I.rpw, I.kc, I.P, I.nw, sm, w, local);
+    if (I.sched == kSchedInOrder && I.rpw == 32) {
+        if constexpr (KT <= 4)
+            strip_solve<T, KT, TR>(A, M.strips[TR ? 1 : 0], R, I.nw, raw, kBatchWarps, s_bad, w, local);
+        __syncthreads();
+        return;
+    }
+    const int ring = I.kc * I.rpw;
+    BlockSmem<T, KT> sm = carve_block_smem<T, KT>(raw, ring, I.kc);
+    reset_block_smem<T, KT>(sm, ring, I.kc);
     __syncthreads();
-    release_block_smem<T, KT>(sm, I.kc);
-    return ok;
+    if (I.sched == kSchedLevel)
+        block_solve_levels<T, KT, TR>(A, R, M.perm, M.iperm, M.lgroups[TR ? 1 : 0], M.nlgroups[TR ? 1 : 0], I.kc,
+                                      I.nw, sm, w, local);
+    else if ((int)(threadIdx.x >> 5) < I.nw)
+        block_solve<T, KT, TR>(A, R, I.rpw, I.kc, I.P, sm, w, local);
+    __syncthreads();
 }
 
 __device__ __forceinline__ unsigned sm_id()
@@ -73,6 +79,7 @@ k_batch(const BatchMat *__restrict__ mats, const BatchItem *__restrict__ items, 
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ int s_next, s_stop;
+    __shared__ int s_bad;
     for (;;) {
         if (threadIdx.x == 0) {
             s_next = (int)atomicAdd(&ctl->ticket, 1ull);
@@ -91,10 +98,10 @@ k_batch(const BatchMat *__restrict__ mats, const BatchItem *__restrict__ items, 
             trace[3 * it + 2] = (long long)sm_id();
         }
         switch (I.KT) {
-        case 1: run_one<T, 1, TR>(M, I, smraw, b, bt, x, w, withhold); break;
-        case 2: run_one<T, 2, TR>(M, I, smraw, b, bt, x, w, withhold); break;
-        case 4: run_one<T, 4, TR>(M, I, smraw, b, bt, x, w, withhold); break;
-        default: run_one<T, 8, TR>(M, I, smraw, b, bt, x, w, withhold); break;
+        case 1: run_one<T, 1, TR>(M, I, smraw, b, bt, x, &s_bad, w, withhold); break;
+        case 2: run_one<T, 2, TR>(M, I, smraw, b, bt, x, &s_bad, w, withhold); break;
+        case 4: run_one<T, 4, TR>(M, I, smraw, b, bt, x, &s_bad, w, withhold); break;
+        default: run_one<T, 8, TR>(M, I, smraw, b, bt, x, &s_bad, w, withhold); break;
         }
         __syncthreads();
         if (trace && threadIdx.x == 0) trace[3 * it + 1] = (long long)now_ns();
@@ -276,6 +283,8 @@ int batch_grid(size_t smem, const DeviceInfo &di)
     cudaFuncSetAttribute(k_batch<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_batch<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_batch<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    strip_stage_batch<float>(nullptr, nullptr, 0, false, nullptr);
+    strip_stage_batch<double>(nullptr, nullptr, 0, false, nullptr);
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch<float, false>, kBatchThreads, smem);
     if (per_sm < 1) per_sm = 1;

@@ -1,22 +1,18 @@
-// Thread-block-local synchronisation-free solve of one system, used by the
-// single-system block mode (solve.cu) and by the batched solve (batch.cu).
+// Thread-block-local synchronisation-free solve of one system with several
+// lanes per row, and the level-ordered one, used by the single-system block
+// mode (solve.cu) and by the batched solve (batch.cu).  (One lane per row:
+// strip.cuh.)
 #pragma once
 
 #include "rows.cuh"
 
 namespace spt {
 
-// Shared-memory layout (dynamic): kc phase barriers, ring of `ring` rows x
-// KT solution values, per-warp coefficient tables and broadcast buffers,
+// Shared-memory layout (dynamic): ring of `ring` rows x KT solution values,
 // ring of row tags (position of the row held by the slot, -1 = empty), ring
-// of chunk tags, counters {ticket, completed prefix}.  The one-lane-per-row
-// path uses the ring, the coefficient tables, the completed-group counter
-// (single-phase) or the barriers (two-phase); the other path uses the tags.
+// of chunk tags, counters {ticket, completed prefix}.
 template <class T, int KT> struct BlockSmem {
-    uint64_t *bar;  // kc phase barriers: group g arrives on bar[g % kc]
     volatile T *xr;
-    T *coef;   // per active warp: [32][32] in-group coefficients
-    T *xbuf;   // per active warp: KT broadcast values
     volatile int *tag;
     volatile int *cdone;
     int *ctr;
@@ -40,7 +36,9 @@ __device__ __forceinline__ int ld_relaxed_cta_smem(const int *p)
 // group resolve through the warp loop, those up to P groups back through the
 // ring tags, older ones are read from global memory (complete by the
 // throttle).  Returns false when a wait gave up.
-template <class T, int KT, bool TR>
+// DIRECT: the values are read in L's own order (the plan's copy in CSC order
+// may be old).
+template <class T, int KT, bool TR, bool DIRECT = false>
 __device__ bool block_solve(const Sys<T> &A, const Rhs<T> &R, int rpw, int kc, int P,
                             const BlockSmem<T, KT> &sm, const Waiter &w, int withhold)
 {
@@ -97,7 +95,7 @@ __device__ bool block_solve(const Sys<T> &A, const Rhs<T> &R, int rpw, int kc, i
                     const int j = RV<T, TR>::col(A, p);
                     const int pj = order_pos<TR>(n, j);
                     const int cj = pj / rpw;
-                    const T vv = RV<T, TR>::val(A, p);
+                    const T vv = DIRECT ? entry_val<T, TR>(A, p) : RV<T, TR>::val(A, p);
                     if (cj == c) {
                         const int gj = pj - base;
                         if (!((fin >> (gj * lpr)) & 1u)) break;
@@ -139,7 +137,7 @@ __device__ bool block_solve(const Sys<T> &A, const Rhs<T> &R, int rpw, int kc, i
                 for (int r = 0; r < KT; ++r) red[r] = acc[r];
                 group_reduce<T, KT>(red, lpr);
                 if (newly && sl == 0) {
-                    const T d = RV<T, TR>::diag(A, a, e);
+                    const T d = DIRECT ? entry_val<T, TR>(A, TR ? a - 1 : e) : RV<T, TR>::diag(A, a, e);
                     const T *bb = R.b + (int64_t)i * R.ld;
                     T *xx = R.x + (int64_t)i * R.ld;
                     volatile T *xrr = sm.xr + (pos % ring) * KT;
@@ -172,10 +170,6 @@ __device__ bool block_solve(const Sys<T> &A, const Rhs<T> &R, int rpw, int kc, i
     }
 }
 
-// Dependency of a row group on an EARLIER group of the same system (block
-// mode), read from the shared-memory ring once its tag is set, or from
-// global memory for groups too old for the ring (complete by the throttle).
-constexpr int kMaxBatch = 8;
 constexpr int kPreload = 16;  // entries of a row loaded before a group's turn
 
 // acc[r] += v * src[r] for r < KT, with 16-byte loads when the layout allows
@@ -212,25 +206,25 @@ __device__ __forceinline__ void store_vec(T *dst, const T (&v)[KT])
     }
 }
 
-// In-group dependencies of a 32-row group, solved in registers.  Lane L
-// holds the scaled candidates t_L = (b_L - sum over earlier groups) / L_LL,
-// coef[s * 32 + L] = L_Ls / L_LL for every in-group dependency s < L (bit s
-// of dmask; other entries of the table are not initialised) and the final
-// x_L = t_L - sum_s coef[s * 32 + L] x_s: 31 steps; step s broadcasts x_s
-// (final once every s' < s was applied) and every lane that depends on row
-// s subtracts its share.
-template <class T, int KT>
-__device__ __forceinline__ void sweep_scalar(T (&t)[KT], unsigned dmask, const T *coef, int lane)
+// In-group dependencies of a 32-row group, solved in registers: lane L holds
+// the scaled candidates t_L = (b_L - sum over earlier groups) / L_LL and the
+// coefficients C_Ls = L_Ls / L_LL of its in-group dependencies s < L (bits of
+// dmask, coefficient coef(s)); x_L = t_L - sum_s C_Ls x_s.  Every step, each
+// lane that still waits takes one dependency that is solved by now; a row is
+// solved when it waits for none.  The number of steps is the group's longest
+// chain counted in multiply-adds (about 5 for a band of 256, 12 for 64), where
+// a sweep over the rows takes 31.
+template <class T, int KT, class Coef>
+__device__ __forceinline__ void group_list(T (&t)[KT], unsigned dmask, Coef coef)
 {
-    const unsigned need = __reduce_or_sync(SPT_FULL_MASK, dmask);
-#pragma unroll
-    for (int s = 0; s < 31; ++s) {
-        // warp-uniform skip of rows nobody depends on; only for wide tiles,
-        // where the step costs more than the branch (a branch stops the
-        // coefficient load from being hoisted onto the previous step)
-        if (KT > 4 && !((need >> s) & 1u)) continue;
-        const bool hit = (dmask >> s) & 1u;
-        const T cf = coef[s * 32 + lane];
+    unsigned rem = dmask;
+    unsigned done = __ballot_sync(SPT_FULL_MASK, rem == 0);
+    while (done != SPT_FULL_MASK) {
+        // (the smallest unsolved row waits for solved rows only)
+        const unsigned av = rem & done;
+        const bool hit = av != 0;
+        const int s = hit ? __ffs(av) - 1 : 0;
+        const T cf = coef(s);
 #pragma unroll
         for (int r = 0; r < KT; ++r) {
             const T xs = __shfl_sync(SPT_FULL_MASK, t[r], s);
@@ -238,292 +232,9 @@ __device__ __forceinline__ void sweep_scalar(T (&t)[KT], unsigned dmask, const T
             // turn independent rows into NaN
             t[r] = hit ? fma(-cf, xs, t[r]) : t[r];
         }
+        rem &= hit ? ~(1u << s) : ~0u;
+        done = __ballot_sync(SPT_FULL_MASK, rem == 0);
     }
-}
-
-// Block-mode solve with one lane per row (groups of 32 rows, dealt to the
-// warps round-robin).  Groups complete in order.  Group c:
-//   1. before any wait: loads its rows' metadata, right-hand sides and first
-//      kPreload entries, builds its in-group coefficient table and applies
-//      the entries older than the shared-memory ring (global memory);
-//   2. waits, then applies the dependencies held in the ring;
-//   3. resolves the in-group dependencies (column sweep) and publishes: ring
-//      values, completion (release), global copy.
-// Single-phase (the batched solve, many blocks per SM): step 2 waits for
-// every group < c on the completed-group counter, which every lane of the
-// warp polls.  Two-phase (TWO, one block on an SM): step 2 waits for the
-// groups <= c-2 only and applies their entries while group c-1 is still
-// being solved; a second wait for group c-1 and its entries precede step 3.
-// Two-phase completion goes through kc shared mbarriers of one arrival
-// each: group g arrives (release) on bar[g % kc], completing that barrier's
-// phase g / kc; a waiting warp is suspended by the hardware instead of
-// polling.  A barrier's next completion (group g + kc) cannot come before
-// the waiters of g (groups g + 1 and g + 2) are done, as kc >= 4.
-// The chain from one completion to the next has no lane-divergent control
-// flow (reconverging a divergent warp costs thousands of cycles on this
-// path): loads use clamped, always-valid indices, stores of unused lanes go
-// to a row of the coefficient table that is never read, selections are
-// arithmetic.
-// Ring slot safety: the slot of group cj is rewritten by group cj + kc only
-// after every group < cj + kc is complete, i.e. after every reader of cj
-// finished.  Global reads: the warp that solved group g stores g's global x
-// (after publishing g) before it publishes its next group, g + nwarps.  A
-// warp starting group c has itself completed c - nwarps, after acquiring
-// the completion of every group < c - nwarps, which covers the global x of
-// every group <= c - 2 nwarps - 1; entries at least kc >= 2 nwarps + 1
-// groups back are therefore read from global memory before the warp waits.
-template <class T, int KT, bool TR, bool TWO>
-__device__ bool block_solve_sweep(const Sys<T> &A, const Rhs<T> &R, int kc, int P, int nwarps,
-                                  const BlockSmem<T, KT> &sm, const Waiter &w, int withhold)
-{
-    (void)P;
-    constexpr int NP = kPreload;
-    const int lane = threadIdx.x & 31;
-    const int n = A.n;
-    const int ring = kc * 32;  // a power of two
-    const int rmask = ring - 1;
-    const int nchunks = (n + 31) / 32;
-    const int kt = R.k;
-    const int wid = threadIdx.x >> 5;
-    T *coef = sm.coef + (size_t)wid * 1024;
-    const T *ring0 = const_cast<const T *>(sm.xr);
-    // row of position q in processing order (clamped into the system)
-    auto row_at = [&](int q) { return q < n ? (TR ? n - 1 - q : q) : (TR ? n - 1 : 0); };
-    // the row extents of a warp's next group are loaded one group ahead, so
-    // that a group's entries are one dependent load away when it starts
-    int a_nx = 0, e_nx = 0;
-    if (wid < nchunks) {
-        const int i0 = row_at(wid * 32 + lane);
-        a_nx = RV<T, TR>::beg(A, i0);
-        e_nx = RV<T, TR>::end(A, i0);
-    }
-    // groups are dealt round-robin: warp w solves w, w + nwarps, ...
-    for (int c = wid; c < nchunks; c += nwarps) {
-        const int base = c * 32;
-        const int pos = base + lane;
-        const bool valid = pos < n;
-        const int i = row_at(pos);
-        // ---- 1. independent of the solution
-        const int a = a_nx;
-        const int e = e_nx;
-        if (c + nwarps < nchunks) {
-            const int inx = row_at(pos + 32 * nwarps);
-            a_nx = RV<T, TR>::beg(A, inx);
-            e_nx = RV<T, TR>::end(A, inx);
-        }
-        const int safe = TR ? a - 1 : e;  // position of the diagonal entry
-        const T rinv = valid ? T(1) / RV<T, TR>::diag(A, a, e) : T(0);
-        T acc[KT], bv[KT];
-#pragma unroll
-        for (int r = 0; r < KT; ++r) {
-            acc[r] = T(0);
-            bv[r] = (valid && r < kt) ? R.b[(int64_t)i * R.ld + r] : T(0);
-        }
-        if (!TR && valid && has_trow(A, i)) {
-            for (int p = A.trp[i]; p < A.trp[i + 1]; ++p) {
-                const T tv = ldro(A.tv + p);
-                const T *bb = R.b + (int64_t)tcol(A, p) * R.ld;
-#pragma unroll
-                for (int r = 0; r < KT; ++r)
-                    if (r < kt) acc[r] -= tv * bb[r];
-            }
-        }
-        int jj[NP];
-        T vv[NP];
-#pragma unroll
-        for (int u = 0; u < NP; ++u) {
-            const int q = a + u < e ? a + u : safe;
-            jj[u] = order_pos<TR>(n, RV<T, TR>::col(A, q));
-            vv[u] = RV<T, TR>::val(A, q);
-        }
-        unsigned dmask = 0;
-#pragma unroll
-        for (int u = 0; u < NP; ++u) {
-            const bool in = valid && a + u < e && jj[u] >= base;
-            coef[(in ? jj[u] - base : 31) * 32 + lane] = vv[u] * rinv;
-            dmask |= in ? (1u << (jj[u] - base)) : 0u;
-        }
-        // entries beyond the first NP (long rows; in the transpose view,
-        // columns longer than NP -- there the farthest entries): in-group
-        // ones go to the table; the others are classified so that only the
-        // rare ones in group c-1 are left for the group's turn
-        const bool longrow = valid && e - a > NP;
-        bool tail_near = false, tail_ring = false;
-        for (int p0 = a + NP; longrow && p0 < e; p0 += 4) {
-            // four entries per round of loads (clamped to the row's last
-            // entry, which exists since p0 < e)
-            int pjs[4];
-            T vs[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int p = min(p0 + q, e - 1);
-                pjs[q] = order_pos<TR>(n, RV<T, TR>::col(A, p));
-                vs[q] = RV<T, TR>::val(A, p);
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                if (p0 + q >= e) break;
-                const int pj = pjs[q];
-                if (pj >= base) {
-                    dmask |= 1u << (pj - base);
-                    coef[(pj - base) * 32 + lane] = vs[q] * rinv;
-                } else if (c - (pj >> 5) < kc) {
-                    if (pj >= base - 32) tail_near = true;
-                    else tail_ring = true;
-                }
-            }
-        }
-        const bool anylong = __any_sync(SPT_FULL_MASK, longrow);
-        bool ok = true;
-        {
-            // entries older than the ring (groups <= c - kc) are read from
-            // global memory now, before the group's turn (see the visibility
-            // argument above)
-            bool any_old = false;
-#pragma unroll
-            for (int u = 0; u < NP; ++u)
-                any_old |= valid && a + u < e && c - (jj[u] >> 5) >= kc;
-            if (__any_sync(SPT_FULL_MASK, any_old)) {
-#pragma unroll
-                for (int u = 0; u < NP; ++u) {
-                    if (valid && a + u < e && c - (jj[u] >> 5) >= kc) {
-                        const T *xx = R.x + (int64_t)order_pos<TR>(n, jj[u]) * R.ld;
-#pragma unroll
-                        for (int r = 0; r < KT; ++r)
-                            if (r < kt) acc[r] += vv[u] * xx[r];
-                    }
-                }
-            }
-            for (int p = a + NP; anylong && longrow && p < e; ++p) {
-                const int j = RV<T, TR>::col(A, p);
-                if (c - (order_pos<TR>(n, j) >> 5) >= kc) {
-                    const T v = RV<T, TR>::val(A, p);
-                    const T *xx = R.x + (int64_t)j * R.ld;
-#pragma unroll
-                    for (int r = 0; r < KT; ++r)
-                        if (r < kt) acc[r] += v * xx[r];
-                }
-            }
-        }
-
-        if constexpr (!TWO) {
-            // the ring pass after the turn is decided now: an entry in the
-            // ring keeps its value and becomes its slot's offset; any other
-            // entry reads slot 0 with weight 0.  Only loads and multiply-adds
-            // are left on the dependent chain.
-#pragma unroll
-            for (int u = 0; u < NP; ++u) {
-                const bool use = valid && a + u < e && jj[u] < base && c - (jj[u] >> 5) < kc;
-                vv[u] = use ? vv[u] : T(0);
-                jj[u] = use ? (jj[u] & rmask) * KT : 0;
-            }
-        }
-        consume(rinv);
-#pragma unroll
-        for (int r = 0; r < KT; ++r) consume(bv[r]);
-        // ---- 2. groups <= c-2 (group g's arrival is phase g / kc of
-        // barrier g % kc); single-phase: all earlier groups (the completed-
-        // group counter reaches c; every lane polls it), after the ring
-        // entries of the row tails that are in groups <= c-2 (waited for
-        // separately, so that their divergent loop runs while group c-1 is
-        // being solved)
-        if constexpr (TWO) {
-            if (c >= 2) ok = mbar_wait(sm.bar + ((c - 2) & (kc - 1)), ((unsigned)(c - 2) / kc) & 1u, w);
-        } else {
-            if (__any_sync(SPT_FULL_MASK, tail_ring)) {
-                WaitClock clk;
-                while (ld_acquire_cta_smem(sm.ctr + 1) < c - 1)
-                    if (clk.expired(w)) { ok = false; break; }
-                if (!__all_sync(SPT_FULL_MASK, ok)) return false;
-                for (int p = a + NP; tail_ring && p < e; ++p) {
-                    const int pj = order_pos<TR>(n, RV<T, TR>::col(A, p));
-                    if (pj < base - 32 && c - (pj >> 5) < kc)
-                        axpy_vec<T, KT>(RV<T, TR>::val(A, p), ring0 + (pj & rmask) * KT, acc);
-                }
-            }
-            // relaxed polls, one acquire fence once the count is reached
-            // (PTX memory model: a relaxed read followed by fence.acq_rel is
-            // an acquire pattern), so that a poll costs one shared load; a
-            // warp two or more groups from its turn sleeps between polls, so
-            // that waiting warps leave the issue slots to the working ones
-            // (several work items share an SM)
-            WaitClock clk;
-            int done;
-            while ((done = ld_relaxed_cta_smem(sm.ctr + 1)) < c) {
-                if (c - done > 1) __nanosleep(200);
-                if (clk.expired(w)) { ok = false; break; }
-            }
-            fence_acq_rel_cta();
-        }
-        if (!__all_sync(SPT_FULL_MASK, ok)) return false;
-        if constexpr (TWO) {
-            const int lim = base - 32;  // ring entries below lim are applied now
-#pragma unroll
-            for (int u = 0; u < NP; ++u) {
-                const bool use = valid && a + u < e && jj[u] < lim && c - (jj[u] >> 5) < kc;
-                axpy_vec<T, KT>(use ? vv[u] : T(0), ring0 + (use ? (jj[u] & rmask) * KT : 0), acc);
-            }
-        } else {
-#pragma unroll
-            for (int u = 0; u < NP; ++u) axpy_vec<T, KT>(vv[u], ring0 + jj[u], acc);
-        }
-        if constexpr (TWO) {
-            if (__any_sync(SPT_FULL_MASK, tail_ring)) {
-                for (int p = a + NP; tail_ring && p < e; ++p) {
-                    const int pj = order_pos<TR>(n, RV<T, TR>::col(A, p));
-                    if (pj < base - 32 && c - (pj >> 5) < kc)
-                        axpy_vec<T, KT>(RV<T, TR>::val(A, p), ring0 + (pj & rmask) * KT, acc);
-                }
-            }
-        } else if (__any_sync(SPT_FULL_MASK, tail_near)) {
-            for (int p = a + NP; tail_near && p < e; ++p) {
-                const int pj = order_pos<TR>(n, RV<T, TR>::col(A, p));
-                if (pj < base && pj >= base - 32)
-                    axpy_vec<T, KT>(RV<T, TR>::val(A, p), ring0 + (pj & rmask) * KT, acc);
-            }
-        }
-        // ---- 3. group c-1 (two-phase), then this group
-        if constexpr (TWO) {
-            if (c >= 1) ok = mbar_wait(sm.bar + ((c - 1) & (kc - 1)), ((unsigned)(c - 1) / kc) & 1u, w);
-            if (!__all_sync(SPT_FULL_MASK, ok)) return false;
-#pragma unroll
-            for (int u = 0; u < NP; ++u) {
-                const bool prev = valid && a + u < e && jj[u] < base && jj[u] >= base - 32;
-                axpy_vec<T, KT>(prev ? vv[u] : T(0), ring0 + (prev ? (jj[u] & rmask) * KT : 0), acc);
-            }
-            if (__any_sync(SPT_FULL_MASK, tail_near)) {
-                for (int p = a + NP; tail_near && p < e; ++p) {
-                    const int pj = order_pos<TR>(n, RV<T, TR>::col(A, p));
-                    if (pj < base && pj >= base - 32)
-                        axpy_vec<T, KT>(RV<T, TR>::val(A, p), ring0 + (pj & rmask) * KT, acc);
-                }
-            }
-        }
-        __syncwarp();
-        T t[KT];
-#pragma unroll
-        for (int r = 0; r < KT; ++r) t[r] = (bv[r] - acc[r]) * rinv;
-        sweep_scalar<T, KT>(t, dmask, coef, lane);
-        // ---- publish: ring values, then (release) the completed-group
-        // counter or, two-phase, the barrier arrival, then the global copy
-        if (valid) store_vec<T, KT>(const_cast<T *>(sm.xr) + (pos & rmask) * KT, t);
-        const bool hold = __any_sync(SPT_FULL_MASK, valid && i == withhold);
-        __syncwarp();
-        if (lane == 0 && !hold) {
-            if constexpr (TWO)
-                mbar_arrive(sm.bar + (c & (kc - 1)));
-            else
-                st_release_cta_smem(sm.ctr + 1, c + 1);
-        }
-        if (valid) {
-            T *xx = R.x + (int64_t)i * R.ld;
-#pragma unroll
-            for (int r = 0; r < KT; ++r)
-                if (r < kt) xx[r] = t[r];
-        }
-        __syncwarp();  // the coefficient table is rewritten by the next group
-    }
-    return true;
 }
 
 // Block-local level-scheduled solve: the rows in level order (transpose:
@@ -698,62 +409,27 @@ __device__ bool block_solve_levels(const Sys<T> &A, const Rhs<T> &R, const int32
     return true;
 }
 
-// Entry used by the kernels: `nwarps` warps of the block work on the system
-// (the others return at once); one lane per row uses the column sweep,
-// two-phase (TWO) or single-phase.
-template <class T, int KT, bool TR, bool TWO>
-__device__ __forceinline__ bool block_solve_any(const Sys<T> &A, const Rhs<T> &R, int rpw, int kc,
-                                                int P, int nwarps, const BlockSmem<T, KT> &sm,
-                                                const Waiter &w, int withhold)
-{
-    if (rpw == 32) {
-        // the sweep's global reads need kc >= 2 nwarps + 1 (always true for
-        // the plans' geometries; enforced here)
-        const int nw = max(1, min(nwarps, (kc - 1) / 2));
-        if ((int)(threadIdx.x >> 5) >= nw) return true;
-        return block_solve_sweep<T, KT, TR, TWO>(A, R, kc, P, nw, sm, w, withhold);
-    }
-    if ((int)(threadIdx.x >> 5) >= nwarps) return true;
-    return block_solve<T, KT, TR>(A, R, rpw, kc, P, sm, w, withhold);
-}
-
 template <class T, int KT>
-__device__ __forceinline__ BlockSmem<T, KT> carve_block_smem(unsigned char *raw, int ring, int kc,
-                                                           int nw)
+__device__ __forceinline__ BlockSmem<T, KT> carve_block_smem(unsigned char *raw, int ring, int kc)
 {
     BlockSmem<T, KT> sm;
-    sm.bar = reinterpret_cast<uint64_t *>(raw);  // kc * 8 bytes keep what follows 16-byte aligned
-    T *xr = reinterpret_cast<T *>(raw + (size_t)kc * 8);
+    T *xr = reinterpret_cast<T *>(raw);
     sm.xr = xr;
-    sm.coef = xr + (size_t)ring * KT;
-    sm.xbuf = sm.coef + (size_t)nw * 1024;
-    int *tag = reinterpret_cast<int *>(sm.xbuf + (size_t)nw * 32);
+    int *tag = reinterpret_cast<int *>(xr + (size_t)ring * KT);
     sm.tag = tag;
     sm.cdone = tag + ring;
     sm.ctr = tag + ring + kc;
     return sm;
 }
 
-// Fresh state for one system (the barriers must not hold a live mbarrier:
-// first use of the memory, or release_block_smem ran).
+// Fresh state for one system.
 template <class T, int KT>
 __device__ __forceinline__ void reset_block_smem(const BlockSmem<T, KT> &sm, int ring, int kc)
 {
     for (int t = threadIdx.x; t < ring * KT; t += blockDim.x) sm.xr[t] = T(0);
     for (int t = threadIdx.x; t < ring; t += blockDim.x) sm.tag[t] = -1;
-    for (int t = threadIdx.x; t < kc; t += blockDim.x) {
-        sm.cdone[t] = -1;
-        mbar_init(sm.bar + t, 1);
-    }
+    for (int t = threadIdx.x; t < kc; t += blockDim.x) sm.cdone[t] = -1;
     if (threadIdx.x == 0) { sm.ctr[0] = 0; sm.ctr[1] = 0; }
-}
-
-// After a __syncthreads that ends the work on one system: invalidate the
-// barriers so that the memory can be re-initialised for the next one.
-template <class T, int KT>
-__device__ __forceinline__ void release_block_smem(const BlockSmem<T, KT> &sm, int kc)
-{
-    for (int t = threadIdx.x; t < kc; t += blockDim.x) mbar_inval(sm.bar + t);
 }
 
 }  // namespace spt

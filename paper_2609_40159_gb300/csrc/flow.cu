@@ -246,12 +246,12 @@ template <class T, bool TR> __global__ void __launch_bounds__(256) k_flow_stage(
         const int llpr = meta_llpr(ln.meta);
         T v[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = s.x + (u << llpr) < s.y ? RV<T, TR>::val(A, s.x + (u << llpr)) : T(0);
+        for (int u = 0; u < 4; ++u) v[u] = s.x + (u << llpr) < s.y ? entry_val<T, TR>(A, s.x + (u << llpr)) : T(0);
         Four<T> f;
         f.set(v);
         f.store(F.vals, t);
         if ((t & ((1 << llpr) - 1)) == 0)
-            static_cast<T *>(F.inv)[t] = T(1) / RV<T, TR>::diag(A, s.x, s.y);
+            static_cast<T *>(F.inv)[t] = T(1) / entry_val<T, TR>(A, TR ? s.x - 1 : s.y);
     }
 }
 
@@ -382,13 +382,13 @@ k_flow(Sys<T> A, FlowSched F, Rhs<T> R, int32_t withhold, Waiter w)
                 const int2 s = F.src[(int64_t)gi * 32 + lane];
                 int p = s.x + 128;
                 uint32_t cn = p < s.y ? ldro(F.ecode + p) : 0u;
-                T vn = p < s.y ? RV<T, TR>::val(A, p) : T(0);
+                T vn = p < s.y ? entry_val<T, TR>(A, p) : T(0);
                 for (; ok && __any_sync(SPT_FULL_MASK, p < s.y); p += 32) {
                     uint32_t c1 = cn;
                     const T v1 = vn;
                     const int pn = p + 32;
                     cn = pn < s.y ? ldro(F.ecode + pn) : 0u;
-                    vn = pn < s.y ? RV<T, TR>::val(A, pn) : T(0);
+                    vn = pn < s.y ? entry_val<T, TR>(A, pn) : T(0);
                     T xf = T(0), x1;
                     const bool old = c1 != 0u && !(c1 & kNear);
                     if (old) {

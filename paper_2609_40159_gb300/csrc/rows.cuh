@@ -36,6 +36,13 @@ template <class T> struct RV<T, true> {
     static __device__ __forceinline__ T val(const Sys<T> &A, int q) { return ldro(A.cv + chk_pos(A, q)); }
 };
 
+// Current value of entry p (the plan's CSC copy of the values is refreshed for
+// other paths only).
+template <class T, bool TR> __device__ __forceinline__ T entry_val(const Sys<T> &A, int p)
+{
+    return TR ? ldro(A.v + chk_pos(A, ldro(A.tmap + chk_pos(A, p)))) : RV<T, false>::val(A, p);
+}
+
 // Column of entry p of T (the rewritten right-hand side's extra terms).
 template <class T> __device__ __forceinline__ int tcol(const Sys<T> &A, int p)
 {

@@ -12,16 +12,17 @@
 //                       its own predecessors' ready flags (ld.acquire /
 //                       st.release), rows of the same group resolve through
 //                       shared memory.
-//   k_block             one thread block per system (one per tile of 8
-//                       right-hand-side columns); recent solutions in a
-//                       shared-memory ring, in-order row groups (for deep,
-//                       narrow systems where the cross-SM round trip
-//                       dominates).
+//   k_block, k_strip    one thread block per tile of right-hand-side columns;
+//                       recent solutions in a shared-memory ring, in-order
+//                       row groups (for deep, narrow systems where the
+//                       cross-SM round trip dominates); several lanes per row,
+//                       or one over prepared strips (strip.cuh).
 //   k_csc_values        L's values in CSC order before a transpose solve.
 // Every kernel handles both L x = b (rows in increasing order) and the
 // adjoint L^T g_b = g_x (rows in decreasing order, reading L through its CSC).
 // A rewritten system L' x = b + T b gathers its T row into the same sum.
 #include "block.cuh"
+#include "strip.cuh"
 
 namespace spt {
 
@@ -349,6 +350,7 @@ k_syncfree(Sys<T> A, Rhs<T> R, int rpw, SyncArgs sy)
 // Sync-free solve with one lane per row: dependencies on earlier groups are
 // waited for through their ready flags, dependencies inside the group are
 // resolved by the column sweep (lane s's solution broadcast at step s).
+constexpr int kMaxBatch = 8;  // entries loaded at a time
 constexpr int kSwThreads = 128;
 constexpr int kSwWarps = kSwThreads / 32;
 
@@ -457,7 +459,8 @@ k_syncfree_sweep(Sys<T> A, Rhs<T> R, SyncArgs sy)
     }
 }
 
-constexpr int kBlockThreads = 512;
+// Several lanes per row.
+constexpr int kBlockThreads = 32 * kMaxBlockWarps;
 
 template <class T, int KT, bool TR>
 __global__ void __launch_bounds__(kBlockThreads)
@@ -470,17 +473,30 @@ k_block(Sys<T> A, Rhs<T> R, int rpw, int kc, int P, int nwarps, SyncArgs sy)
     R.x += r0;
     R.k = min(KT, R.k - r0);
     const int ring = kc * rpw;
-    BlockSmem<T, KT> sm = carve_block_smem<T, KT>(smraw, ring, kc, nwarps);
+    BlockSmem<T, KT> sm = carve_block_smem<T, KT>(smraw, ring, kc);
     reset_block_smem<T, KT>(sm, ring, kc);
     __syncthreads();
-    block_solve_any<T, KT, TR, true>(A, R, rpw, kc, P, nwarps, sm, sy.w, sy.withhold);
+    if ((int)(threadIdx.x >> 5) < nwarps) block_solve<T, KT, TR>(A, R, rpw, kc, P, sm, sy.w, sy.withhold);
 }
 
-size_t block_smem_bytes(int rpw, int kt, int kc, bool f64, int nw)
+// One lane per row, over the strips: one block per KT columns.
+template <class T, int KT, bool TR>
+__global__ void __launch_bounds__(32 * kStripWarps)
+k_strip(Sys<T> A, Strips V, Rhs<T> R, SyncArgs sy)
+{
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ int s_bad;
+    const int r0 = blockIdx.x * KT;
+    R.b += r0;
+    R.x += r0;
+    R.k = min(KT, R.k - r0);
+    strip_solve<T, KT, TR>(A, V, R, kStripWarps, smraw, kStripWarps, &s_bad, sy.w, sy.withhold);
+}
+
+size_t block_smem_bytes(int rpw, int kt, int kc, bool f64)
 {
     const size_t ring = (size_t)kc * rpw;
-    const size_t w = f64 ? 8 : 4;
-    return (size_t)kc * 8 + ring * kt * w + (size_t)nw * (1024 + 32) * w + ring * 4 + (size_t)kc * 4 + 16;
+    return ring * kt * (f64 ? 8 : 4) + ring * 4 + (size_t)kc * 4 + 16;
 }
 // ------------------------------------------------------------- gradient
 template <class T>
@@ -672,20 +688,17 @@ void block_geometry(int rpw, int kt, bool f64, int nwarps, int *kc, int *P, size
     // ring shrinks; correctness only needs kc >= 2P >= 2.
     int k = 4;
     while (k < 2 * (nwarps + 2)) k <<= 1;
-    while (k > 4 && block_smem_bytes(rpw, kt, k, f64, nwarps) > kBlockSmemBudget) k >>= 1;
+    while (k > 4 && block_smem_bytes(rpw, kt, k, f64) > kBlockSmemBudget) k >>= 1;
     *P = k / 2;
-    while (k < 4096 / rpw && block_smem_bytes(rpw, kt, k * 2, f64, nwarps) <= grow_limit)
+    while (k < 4096 / rpw && block_smem_bytes(rpw, kt, k * 2, f64) <= grow_limit)
         k <<= 1;  // a longer ring keeps more dependencies in shared memory
     *kc = k;
 }
 
 int block_warps_for(double rows_per_level, int rpw)
 {
-    // one lane per row (column sweep, groups complete in order): the extra
-    // warps preload later groups, so use all of them
-    if (rpw == 32) return kMaxBlockWarps;
     // enough row groups in flight to cover about two levels; at least two
-    // warps so that one group's loads overlap the previous group's sweep
+    // warps so that one group's loads overlap the previous group's
     int w = (int)(2.0 * rows_per_level / rpw + 0.999);
     if (w < 2) w = 2;
     if (w > kMaxBlockWarps) w = kMaxBlockWarps;
@@ -709,7 +722,7 @@ static cudaError_t blk_launch(const Sys<T> &A, const Rhs<T> &R, int rpw, bool tr
 {
     int kc, P;
     block_geometry(rpw, KT, sizeof(T) == 8, nwarps, &kc, &P, kBlockSmemBudget / 2);
-    const size_t smem = block_smem_bytes(rpw, KT, kc, sizeof(T) == 8, nwarps);
+    const size_t smem = block_smem_bytes(rpw, KT, kc, sizeof(T) == 8);
     if (smem > kBlockSmemBudget) return cudaErrorInvalidConfiguration;
     const int tiles = (R.k + KT - 1) / KT;
     if (trans) {
@@ -722,8 +735,25 @@ static cudaError_t blk_launch(const Sys<T> &A, const Rhs<T> &R, int rpw, bool tr
     return cudaGetLastError();
 }
 
-// Columns per thread block: the next power of two up to 8; wider right-hand
-// sides run as several blocks of 8 columns.
+template <class T, int KT>
+static cudaError_t strip_launch(const Sys<T> &A, const Strips &V, const Rhs<T> &R, bool trans, const SyncArgs &sy,
+                                cudaStream_t s)
+{
+    const size_t smem = strip_smem(V.ring, KT, sizeof(T) == 8, kStripWarps);
+    if (smem > kBlockSmemBudget) return cudaErrorInvalidConfiguration;
+    const int tiles = (R.k + KT - 1) / KT;
+    if (trans) {
+        raise_smem_once<k_strip<T, KT, true>>();
+        k_strip<T, KT, true><<<tiles, 32 * kStripWarps, smem, s>>>(A, V, R, sy);
+    } else {
+        raise_smem_once<k_strip<T, KT, false>>();
+        k_strip<T, KT, false><<<tiles, 32 * kStripWarps, smem, s>>>(A, V, R, sy);
+    }
+    return cudaGetLastError();
+}
+
+// Columns per thread block of the several-lanes kernel: the next power of two
+// up to 8; wider right-hand sides run as several blocks of 8 columns.
 int block_kt_for(int k)
 {
     int kt = 1;
@@ -737,16 +767,24 @@ bool block_mode_supported(int k, bool f64)
     const int kt = block_kt_for(k);
     int kc, P;
     block_geometry(32, kt, f64, kMaxBlockWarps, &kc, &P, kBlockSmemBudget / 2);
-    return block_smem_bytes(32, kt, kc, f64, kMaxBlockWarps) <= kBlockSmemBudget;
+    return block_smem_bytes(32, kt, kc, f64) <= kBlockSmemBudget;
 }
 
 template <class T>
-cudaError_t solve_block(const Sys<T> &A, const Rhs<T> &R, int rpw, int kt, bool trans,
+cudaError_t solve_block(const Sys<T> &A, const Strips &V, const Rhs<T> &R, int rpw, bool trans,
                         const SyncArgs &sy, int nwarps, cudaStream_t s)
 {
-    (void)kt;
     cudaError_t e = launch_prologue<T>(sy.ctl, s);
+    if (e == cudaSuccess && rpw == 32) e = strip_stage<T>(A, V, trans, s);
     if (e != cudaSuccess || A.n <= 0) return e;
+    if (rpw == 32) {
+        // the columns are independent chains, and a block's chain grows with
+        // its columns: one each while there is an SM for it (every block reads
+        // the staged system, which L2 serves)
+        if (R.k <= 152) return strip_launch<T, 1>(A, V, R, trans, sy, s);
+        if (R.k <= 304) return strip_launch<T, 2>(A, V, R, trans, sy, s);
+        return strip_launch<T, 4>(A, V, R, trans, sy, s);
+    }
     switch (block_kt_for(R.k)) {
     case 1: return blk_launch<T, 1>(A, R, rpw, trans, sy, nwarps, s);
     case 2: return blk_launch<T, 2>(A, R, rpw, trans, sy, nwarps, s);
@@ -838,7 +876,7 @@ cudaError_t csc_values(const int32_t *tmap, const T *v, T *cv, int64_t nnz, cuda
                                                    int, bool, const SyncArgs &, int, cudaStream_t);     \
     template cudaError_t solve_syncfree<T>(const Sys<T> &, const Rhs<T> &, int, int, bool,              \
                                            const SyncArgs &, int, cudaStream_t);                        \
-    template cudaError_t solve_block<T>(const Sys<T> &, const Rhs<T> &, int, int, bool,                 \
+    template cudaError_t solve_block<T>(const Sys<T> &, const Strips &, const Rhs<T> &, int, bool,      \
                                         const SyncArgs &, int, cudaStream_t);                           \
     template cudaError_t grad_vals<T>(const Sys<T> &, const T *, const T *, int64_t, int32_t, T *,      \
                                       cudaStream_t);                                                    \

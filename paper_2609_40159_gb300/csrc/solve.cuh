@@ -70,6 +70,23 @@ struct SyncArgs {
     unsigned long long *vflags = nullptr;
 };
 
+// ------------------------------------------------------------------ strips
+// (strip.cuh)
+constexpr int kStripNear = 16, kStripOld = 28;  // staged dependencies a row: on the previous group, older ones
+
+// Kinds of a group's in-group dependencies.
+constexpr uint32_t kTriNone = 0;     // none
+constexpr uint32_t kTriSteps = 1;    // a schedule of steps, one dependency of every row each
+constexpr uint32_t kTriInverse = 2;  // FP32, many: product with the inverse triangle
+
+// Strips of one system and direction: a block of bytes for every group.
+struct Strips {
+    unsigned char *blocks;  // null: not built
+    const uint32_t *ofs;    // start of every group's block, in units of 16 bytes; the end
+    const uint16_t *ecode;  // by entry: where its value goes (strip.cu)
+    int32_t ring;           // rows of a column's ring of solutions
+};
+
 // ---------------------------------------------------------------- launchers
 // All return cudaSuccess or the launch error; T = double or float.
 template <class T>
@@ -89,8 +106,9 @@ template <class T>
 cudaError_t solve_syncfree(const Sys<T> &A, const Rhs<T> &R, int rpw, int kt, bool trans,
                            const SyncArgs &sy, int grid, cudaStream_t s);
 
+// V: the direction's strips (rpw == 32), refreshed by the call.
 template <class T>
-cudaError_t solve_block(const Sys<T> &A, const Rhs<T> &R, int rpw, int kt, bool trans,
+cudaError_t solve_block(const Sys<T> &A, const Strips &V, const Rhs<T> &R, int rpw, bool trans,
                         const SyncArgs &sy, int nwarps, cudaStream_t s);
 
 template <class T>
@@ -119,16 +137,22 @@ int block_kt_for(int k);
 void block_geometry(int rpw, int kt, bool f64, int nwarps, int *kc, int *P, size_t grow_limit);
 // Active warps of the block mode for a system with the given level width.
 int block_warps_for(double rows_per_level, int rpw);
-size_t block_smem_bytes(int rpw, int kt, int kc, bool f64, int nw);
+size_t block_smem_bytes(int rpw, int kt, int kc, bool f64);
 // Most warps of a block-mode thread block that work on one system.
 constexpr int kMaxBlockWarps = 8;
 // Batched solve: warps per thread block and the minimum number of resident
 // blocks per SM the kernel is compiled for (0 = no register constraint).
 constexpr int kBatchWarps = 4;
-constexpr int kBatchMinBlocks = 0;
+constexpr int kBatchMinBlocks = 2;
 // Shared memory a batched work item may grow its ring to: several items per
 // SM (each a latency-bound chain) beat longer rings.
 constexpr size_t kBatchSmemGrow = 48 * 1024;
+// Rows of a column's ring of solutions over the strips (older solutions are
+// read from global memory, at least 2 kMaxBlockWarps + 1 groups back): most,
+// for single systems and batches (four columns a block; byte offsets in the
+// ring fit 16 bits; four blocks of a batch on an SM).
+constexpr int kStripRingLeast = 32 * (2 * kMaxBlockWarps + 2);
+constexpr int strip_ring_most(bool f64, bool batched) { return batched ? (f64 ? 608 : 1216) : (f64 ? 1536 : 3072); }
 constexpr size_t kBlockSmemBudget = 200 * 1024;
 
 // ---------------------------------------------------------------- batched
@@ -163,6 +187,7 @@ struct BatchMat {
     const int32_t *perm, *iperm;
     const LevelGroup *lgroups[2];
     int32_t nlgroups[2];
+    Strips strips[2];  // per direction, for items in row order with one lane per row
 };
 
 // Schedules of a batched work item.
