@@ -699,7 +699,11 @@ sptrsv_status solve_impl(sptrsv_plan p, const void *b, void *x, int32_t nrhs, in
     // schedules that lay the values out themselves
     const bool strips = mode == SPTRSV_MODE_BLOCK && p->rpw == 32 && M.strips[dir].blocks != nullptr;
     const bool flow = mode == SPTRSV_MODE_HYBRID && use_flow(p, dir);
-    if (trans && !strips && !flow) {
+    // (k_level_cols fills x before it reads b)
+    const size_t span = ((size_t)(M.L.n - 1) * (size_t)ld + (size_t)nrhs) * sizeof(T);
+    const bool apart = (const char *)b + span <= (const char *)x || (const char *)x + span <= (const char *)b;
+    const bool cols = mode == SPTRSV_MODE_LEVEL_PERSISTENT && p->rpw == 32 && apart;
+    if (trans && !strips && !flow && !cols) {
         cudaError_t eg = csc_values<T>(M.d_tmap, (const T *)M.L.vals, (T *)M.d_cv, M.L.nnz, s);
         if (eg != cudaSuccess) return from_cuda(eg);
     }
@@ -718,6 +722,10 @@ sptrsv_status solve_impl(sptrsv_plan p, const void *b, void *x, int32_t nrhs, in
         if (st != SPTRSV_OK) return st;
         Sched S{M.d_perm, M.d_level_ptr, M.nlevels, trans ? p->d_chunk_tr : p->d_chunk_fwd,
                 ((int64_t)M.L.n + p->rpw - 1) / p->rpw};
+        if (cols) {
+            e = solve_level_cols<T>(A, S, R, kt, trans, sy, p->grid_level, s);
+            break;
+        }
         const int64_t want = (2 * (int64_t)p->max_width / p->rpw + 7) / 8;  // blocks of 8 warps
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(p->grid_level, want));
         e = solve_level_persistent<T>(A, S, R, p->rpw, kt, trans, sy, grid, s);

@@ -8,6 +8,8 @@
 //                       a ticket and wait on a grid-wide progress counter
 //                       (rows of all earlier levels done) instead of a launch
 //                       boundary.
+//   k_level_cols        the same order, one lane per row and column, waiting
+//                       on the solutions themselves (32 rows per warp).
 //   k_syncfree          one launch; row groups in row order; each row waits on
 //                       its own predecessors' ready flags (ld.acquire /
 //                       st.release), rows of the same group resolve through
@@ -231,6 +233,201 @@ k_level_persistent(Sys<T> A, Sched S, Rhs<T> R, int rpw, SyncArgs sy)
             if (hi >= q1) break;
             ++l;
         }
+    }
+}
+
+// Level order with one lane per row and column, every solution its own flag:
+// x is filled with a NaN that no solution has, and a lane polls the solutions
+// that its row depends on until they are there, so a level costs one hop
+// through L2 (store to poll) instead of those of a fence, a counter and a load.
+// The KT lanes of a row read its entries once and its dependencies side by
+// side.  Everything else (entries, reciprocal diagonals, right-hand sides) is
+// loaded before, with enough blocks resident that this happens levels ahead;
+// values are read in L's own order, so a transpose needs no copy in CSC order.
+// Chunks are taken from a ticket in level order, so what a chunk waits for is
+// done or running; a count of finished rows, read before the first poll, keeps
+// blocks more than four levels ahead from polling.
+// 128^3 Laplacian, 8 columns, FP64 (382 levels of 5,500 rows): 0.73 ms a solve;
+// 3.3 ms with one lane per row for all columns, loads after the wait and a
+// counter of finished rows; 2.2 ms with this layout and that counter.
+template <class T> struct Unsolved;
+template <> struct Unsolved<float> {
+    using Bits = uint32_t;
+    static constexpr Bits mark = 0x7fc5a3c7u, other = 0x7fffffffu;
+    static __device__ __forceinline__ Bits load(const float *p)
+    {
+        Bits v;
+        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+        return v;
+    }
+    static __device__ __forceinline__ void store(float *p, float x)
+    {
+        Bits v = __float_as_uint(x);
+        v = v == mark ? other : v;
+        asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+    }
+    static __device__ __forceinline__ float value(Bits v) { return __uint_as_float(v); }
+};
+template <> struct Unsolved<double> {
+    using Bits = unsigned long long;
+    static constexpr Bits mark = 0x7ff85a5aa5a53c3cull, other = 0x7fffffffffffffffull;
+    static __device__ __forceinline__ Bits load(const double *p)
+    {
+        Bits v;
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+        return v;
+    }
+    static __device__ __forceinline__ void store(double *p, double x)
+    {
+        Bits v = (Bits)__double_as_longlong(x);
+        v = v == mark ? other : v;
+        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+    }
+    static __device__ __forceinline__ double value(Bits v) { return __longlong_as_double((long long)v); }
+};
+
+template <class T> __global__ void __launch_bounds__(256) k_unsolved(T *x, int64_t total, int64_t ld, int32_t k)
+{
+    using U = Unsolved<T>;
+    auto *xb = reinterpret_cast<typename U::Bits *>(x);
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
+         t += (int64_t)gridDim.x * blockDim.x) {
+        if (ld == k) {
+            xb[t] = U::mark;
+        } else {
+            const int64_t i = t / k;
+            xb[i * ld + (t - i * k)] = U::mark;
+        }
+    }
+}
+
+__host__ __device__ constexpr int cols_threads(int KT) { return KT >= 8 ? 256 : 128; }
+
+// E: entries of a row in registers at a time.  Rows of four dependencies in the
+// mean take E = 4 and five blocks of 256 threads an SM (0.73 ms in the case
+// above; E = 8: 1.08 ms; six blocks, with spills: 0.77 ms), longer ones E = 8
+// and four (100 levels of 4,000 random rows of 6 entries, FP64, 8 columns:
+// 0.49 ms against 0.80 with five).
+template <class T, int KT, int E, bool TR>
+__global__ void __launch_bounds__(cols_threads(KT), (E == 4 ? 1280 : 1024) / cols_threads(KT))
+k_level_cols(Sys<T> A, Sched S, Rhs<T> R, SyncArgs sy)
+{
+    using U = Unsolved<T>;
+    constexpr int RB = cols_threads(KT) / KT;
+    __shared__ unsigned long long s_c[2];
+    __shared__ int s_fail;
+    __shared__ T s_rinv[RB];
+    const int g = threadIdx.x / KT, col = threadIdx.x % KT;
+    const int n = A.n, L = S.nlevels;
+    auto start_of = [&](int l) { return TR ? n - S.level_ptr[L - l] : S.level_ptr[l]; };
+    auto row_of = [&](int q) { return chk_row(A, TR ? S.perm[n - 1 - q] : S.perm[q]); };
+    if (threadIdx.x == 0) {
+        s_c[0] = atomicAdd(&sy.ctl->ticket, 1ull);
+        s_fail = 0;
+    }
+    int rows = 0;  // of the chunk before
+    for (int it = 0;; it ^= 1) {
+        __syncthreads();
+        if (threadIdx.x == 0 && rows > 0) atomicAdd(&sy.ctl->progress, (unsigned long long)rows);
+        const unsigned long long c = s_c[it];
+        if (s_fail || c >= ((unsigned long long)n + RB - 1) / RB) return;
+        const int q0 = (int)c * RB, q = q0 + g;
+        rows = min(RB, n - q0);
+        if (threadIdx.x == 0) s_c[it ^ 1] = atomicAdd(&sy.ctl->ticket, 1ull);
+        // reciprocals once a row (an FP64 division takes a warp as long as
+        // twelve multiply-adds, whatever its lanes share)
+        if (threadIdx.x < RB && q0 + (int)threadIdx.x < n) {
+            const int i = row_of(q0 + threadIdx.x);
+            s_rinv[threadIdx.x] = T(1) / entry_val<T, TR>(A, TR ? RV<T, TR>::beg(A, i) - 1 : RV<T, TR>::end(A, i));
+        }
+        const bool active = q < n;
+        const int i = active ? row_of(q) : 0;
+        const int a = active ? RV<T, TR>::beg(A, i) : 0;
+        const int e = active ? RV<T, TR>::end(A, i) : 0;
+        int jj[E];
+        T vv[E], bv = T(0), acc = T(0);
+        auto take_entries = [&](int p) {
+#pragma unroll
+            for (int u = 0; u < E; ++u) {
+                jj[u] = 0;
+                vv[u] = T(0);
+                if (p + u < e) {
+                    jj[u] = RV<T, TR>::col(A, p + u);
+                    vv[u] = entry_val<T, TR>(A, p + u);
+                }
+            }
+        };
+        auto take_rhs = [&](int r) {
+            const bool mine = active && r < R.k;
+            bv = mine ? R.b[(int64_t)i * R.ld + r] : T(0);
+            acc = T(0);
+            if (!TR && mine && has_trow(A, i))
+                for (int p = A.trp[i]; p < A.trp[i + 1]; ++p)
+                    acc -= ldro(A.tv + p) * R.b[(int64_t)tcol(A, p) * R.ld + r];
+        };
+        take_entries(a);
+        take_rhs(col);
+        consume(bv);
+        consume(acc);
+#pragma unroll
+        for (int u = 0; u < E; ++u) consume(vv[u]);
+        bool ok = true;
+        if (threadIdx.x == 0) {
+            int l = S.chunk_level[q0 / 32];  // (of the 32 rows that q0 is one of)
+            while (start_of(l + 1) <= q0) ++l;
+            const unsigned long long from = (unsigned long long)start_of(max(l - 4, 0));
+            WaitClock clk;
+            while (ld_relaxed_u64(&sy.ctl->progress) < from) {
+                if (clk.expired(sy.w)) { ok = false; break; }
+                __nanosleep(32);
+            }
+        }
+        if (!__syncthreads_and(ok)) return;
+        const T rinv = s_rinv[g];
+        bool failed = false;
+        for (int r0 = 0; r0 < R.k && !failed; r0 += KT) {
+            const int r = r0 + col;
+            const T *xr = R.x + r;
+            if (r0 > 0) {
+                take_rhs(r);
+                if (e - a > E) take_entries(a);
+            }
+            bool open = active && r < R.k;
+            int p = a;
+            unsigned pend = (1u << min(max(e - p, 0), E)) - 1u;
+            typename U::Bits xv[E];
+            WaitClock clk;
+            for (;;) {
+                if (open) {
+#pragma unroll
+                    for (int u = 0; u < E; ++u)
+                        if ((pend >> u) & 1u) xv[u] = U::load(xr + (int64_t)jj[u] * R.ld);
+#pragma unroll
+                    for (int u = 0; u < E; ++u)
+                        if (((pend >> u) & 1u) && xv[u] != U::mark) pend &= ~(1u << u);
+                    if (pend == 0) {
+#pragma unroll
+                        for (int u = 0; u < E; ++u)
+                            if (p + u < e) acc += vv[u] * U::value(xv[u]);
+                        p += E;
+                        if (p < e) {
+                            take_entries(p);
+                            pend = (1u << min(e - p, E)) - 1u;
+                        } else {
+                            // (test hook: a withheld row is never published)
+                            if (i != sy.withhold) U::store(R.x + (int64_t)i * R.ld + r, (bv - acc) * rinv);
+                            open = false;
+                        }
+                    }
+                }
+                if (!__any_sync(SPT_FULL_MASK, open)) break;
+                if (__any_sync(SPT_FULL_MASK, clk.expired(sy.w))) {
+                    failed = true;
+                    break;
+                }
+            }
+        }
+        if (failed) s_fail = 1;
     }
 }
 
@@ -633,6 +830,39 @@ static cudaError_t lp_launch(const Sys<T> &A, const Sched &S, const Rhs<T> &R, i
     return cudaGetLastError();
 }
 
+template <class T, int KT>
+static cudaError_t lc_launch(const Sys<T> &A, const Sched &S, const Rhs<T> &R, bool trans, const SyncArgs &sy,
+                             int grid, cudaStream_t s)
+{
+    constexpr int threads = cols_threads(KT), RB = threads / KT;
+    const int64_t total = (int64_t)A.n * R.k;
+    k_unsolved<T><<<(int)std::min<int64_t>((total + 255) / 256, 152 * 8), 256, 0, s>>>(R.x, total, R.ld, R.k);
+    // (four blocks of 128 threads an SM: with all six, 480 us where four take
+    // 395, 128^3 Laplacian, FP32, one column)
+    if (threads == 128) grid = grid - grid / 3;
+    grid = (int)std::min<int64_t>(grid, ((int64_t)A.n + RB - 1) / RB);
+    const bool few = A.nnz <= 5 * (int64_t)A.n;
+    auto *k = trans ? (few ? k_level_cols<T, KT, 4, true> : k_level_cols<T, KT, 8, true>)
+                    : (few ? k_level_cols<T, KT, 4, false> : k_level_cols<T, KT, 8, false>);
+    k<<<grid, threads, 0, s>>>(A, S, R, sy);
+    return cudaGetLastError();
+}
+
+template <class T>
+cudaError_t solve_level_cols(const Sys<T> &A, const Sched &S, const Rhs<T> &R, int kt, bool trans,
+                             const SyncArgs &sy, int grid, cudaStream_t s)
+{
+    cudaError_t e = launch_prologue<T>(sy.ctl, s);
+    if (e != cudaSuccess || A.n <= 0) return e;
+    switch (kt) {
+    case 1: return lc_launch<T, 1>(A, S, R, trans, sy, grid, s);
+    case 2: return lc_launch<T, 2>(A, S, R, trans, sy, grid, s);
+    case 4: return lc_launch<T, 4>(A, S, R, trans, sy, grid, s);
+    case 8: return lc_launch<T, 8>(A, S, R, trans, sy, grid, s);
+    default: return lc_launch<T, 16>(A, S, R, trans, sy, grid, s);
+    }
+}
+
 template <class T>
 cudaError_t solve_level_persistent(const Sys<T> &A, const Sched &S, const Rhs<T> &R, int rpw,
                                    int kt, bool trans, const SyncArgs &sy, int grid, cudaStream_t s)
@@ -872,6 +1102,8 @@ cudaError_t csc_values(const int32_t *tmap, const T *v, T *cv, int64_t nnz, cuda
     template cudaError_t solve_level_launch<T>(const Sys<T> &, const int32_t *,                         \
                                                const std::vector<int32_t> &, const Rhs<T> &, bool,     \
                                                cudaStream_t);                                           \
+    template cudaError_t solve_level_cols<T>(const Sys<T> &, const Sched &, const Rhs<T> &, int, bool,   \
+                                             const SyncArgs &, int, cudaStream_t);                      \
     template cudaError_t solve_level_persistent<T>(const Sys<T> &, const Sched &, const Rhs<T> &, int, \
                                                    int, bool, const SyncArgs &, int, cudaStream_t);     \
     template cudaError_t solve_syncfree<T>(const Sys<T> &, const Rhs<T> &, int, int, bool,              \

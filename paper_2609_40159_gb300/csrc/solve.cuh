@@ -102,6 +102,11 @@ cudaError_t solve_level_persistent(const Sys<T> &A, const Sched &S, const Rhs<T>
                                    int kt, bool trans, const SyncArgs &sy, int grid,
                                    cudaStream_t s);
 
+// S.chunk_level: of 32-row groups.
+template <class T>
+cudaError_t solve_level_cols(const Sys<T> &A, const Sched &S, const Rhs<T> &R, int kt, bool trans,
+                             const SyncArgs &sy, int grid, cudaStream_t s);
+
 template <class T>
 cudaError_t solve_syncfree(const Sys<T> &A, const Rhs<T> &R, int rpw, int kt, bool trans,
                            const SyncArgs &sy, int grid, cudaStream_t s);
