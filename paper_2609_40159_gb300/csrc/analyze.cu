@@ -72,13 +72,24 @@ constexpr int kLevThreads = 256;
 constexpr int kLevWarps = kLevThreads / 32;
 
 constexpr int kLevLong = 32;  // rows with more off-diagonals are walked by the whole warp
+// Entries of a row that are looked at together, and the longest pause between
+// looks (ns).  A row waits for the last of its dependencies, and those before
+// it cost a round trip each when they are looked at one by one: band of 64,
+// 300,000 rows of 4-16 entries 80.2 -> 27.4 ms, power-law 1M 41.5 ->
+// 27.1 ms, band of 1,024 10.6 -> 7.1 ms.  Eight at a time: 24, 28 and 7.2
+// ms, but lap2d 1024^2 2.6 -> 2.8 ms (fewer warps resident).  A row that has
+// seen nothing new looks at its next dependency only (the warps far ahead of the
+// wavefront would take L2's bandwidth from it: band of 1,024 9.9 ms instead of
+// 7.0); pauses of up to 256 ns give 7.0 / 26.0 / 2.6 ms but cost a chain 7 %.
+constexpr int kLevLook = 4;
+constexpr int kLevPause = 128;
 
 // Levels by a synchronisation-free pass over chunks of 32 consecutive rows,
 // taken by warps from a ticket: a chunk only waits on chunks already taken
 // by running warps, so the pass needs no co-residency.  A level is its own
 // ready flag (-1 until published, read with relaxed loads).  A chunk works
-// in rounds: every row polls its dependencies on earlier chunks without
-// blocking (a cursor stops at the first one not yet published); a row
+// in rounds: every row polls its dependencies on earlier chunks, a few at a
+// time, without blocking; a row
 // whose earlier-chunk dependencies are all seen and whose dependencies in
 // the chunk are all published takes its level at once (the chunk's levels
 // are kept in shared memory), so that rows are published as early as
@@ -110,23 +121,43 @@ k_levels(const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, int32_t
         unsigned dmask = 0;     // dependencies on rows of this chunk
         bool ext = !valid || (!islong && a >= pend);  // every earlier-chunk dependency seen
         bool pub = !valid;      // level published (or withheld by the test hook)
+        // entries [p - kLevLook, p) are looked at together; those not yet published
+        // are left
+        int jw[kLevLook];
+        unsigned left = 0;
+        auto take = [&]() {
+            left = 0;
+#pragma unroll
+            for (int u = 0; u < kLevLook; ++u) {
+                const int j = p + u < pend ? ldro(ci + p + u) : -1;
+                jw[u] = j;
+                if (j >= base) dmask |= 1u << (j - base);
+                else if (j >= 0) left |= 1u << u;
+            }
+            p += kLevLook;
+        };
+        int idle = 0;
         WaitClock clk;
         for (;;) {
             bool moved = false;
             // ---- 1. earlier-chunk dependencies, without blocking
-            while (!ext && !islong && p < pend) {
-                const int32_t j = ldro(ci + p);
-                if (j >= base) {
-                    dmask |= 1u << (j - base);
-                } else {
-                    const int lj = ld_relaxed(lev + j);
-                    if (lj < 0) break;
-                    m = m > lj ? m : lj;
+            while (!ext && !islong) {
+                int lj[kLevLook];
+                const unsigned look = idle > 0 ? left & (0u - left) : left;
+#pragma unroll
+                for (int u = 0; u < kLevLook; ++u) lj[u] = (look >> u) & 1u ? ld_relaxed(lev + jw[u]) : -1;
+                const unsigned before = left;
+#pragma unroll
+                for (int u = 0; u < kLevLook; ++u) {
+                    if (lj[u] >= 0) left &= ~(1u << u);
+                    m = m > lj[u] ? m : lj[u];
                 }
-                ++p;
+                moved |= left != before;
+                if (left) break;
+                if (p >= pend) { ext = true; break; }
+                take();
                 moved = true;
             }
-            if (!islong && p >= pend) ext = true;
             unsigned pending = __ballot_sync(SPT_FULL_MASK, islong && !ext);
             while (pending) {
                 const int s = __ffs(pending) - 1;
@@ -186,7 +217,13 @@ k_levels(const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, int32_t
             }
             // one decision for the whole warp (the lanes' clocks may straddle
             // the limit)
-            if (!__any_sync(SPT_FULL_MASK, moved) && __any_sync(SPT_FULL_MASK, clk.expired(w))) return;
+            if (!__any_sync(SPT_FULL_MASK, moved)) {
+                if (__any_sync(SPT_FULL_MASK, clk.expired(w))) return;
+                ++idle;
+                if (idle > 4) __nanosleep(min(kLevPause, 16 << min(idle - 4, 6)));
+            } else {
+                idle = 0;
+            }
         }
     }
 }
