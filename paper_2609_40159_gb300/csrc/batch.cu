@@ -108,28 +108,14 @@ k_batch(const BatchMat *__restrict__ mats, const BatchItem *__restrict__ items, 
     }
 }
 
-// Row of nonzero p inside a 32-row chunk whose lanes hold the chunk's row
-// starts (s = row_ptr[r0 + lane], lanes >= nrows unused): the last lane l <
-// nrows with s_l <= p, by a five-step binary search over the lanes.
-__device__ __forceinline__ int row_in_chunk(int s, int nrows, int p)
-{
-    int lo = 0;
-#pragma unroll
-    for (int step = 16; step >= 1; step >>= 1) {
-        const int cand = lo + step;
-        const int v = __shfl_sync(SPT_FULL_MASK, s, cand & 31);
-        if (cand < nrows && v <= p) lo = cand;
-    }
-    return lo;
-}
-
 // dL/dL_ij = -g_b[i,:] . x[j,:] on L's pattern.  One warp per 32-row chunk;
 // the chunk's nonzeros are contiguous in CSR order and are taken 32 at a
 // time, one per lane (coalesced column indices and gradient stores).
 // (Groups of up to 8 lanes per nonzero, reading g_b[i,:] and x[j,:] in
 // contiguous pieces, measured slower on the batched workload; so did groups
 // of up to 32 lanes walking the chunk's rows: 8.4 ms instead of 3.0 ms for
-// T^T and the gradient, the extra instructions outweighing the coalescing.)
+// T^T and the gradient, the extra instructions outweighing the coalescing;
+// 16-byte loads where the columns allow: no change.)
 template <class T>
 __global__ void k_batch_grad(const BatchMat *__restrict__ mats, const RowChunk *__restrict__ chunks,
                              int64_t nchunks, const T *__restrict__ gb, const T *__restrict__ x,

@@ -65,6 +65,45 @@ __device__ __forceinline__ void consume(int v) { asm volatile("" ::"r"(v)); }
 __device__ __forceinline__ void consume(float v) { asm volatile("" ::"f"(v)); }
 __device__ __forceinline__ void consume(double v) { asm volatile("" ::"d"(v)); }
 
+// Row of nonzero p inside a 32-row chunk whose lanes hold the chunk's row
+// starts (s = row_ptr[r0 + lane], lanes >= nrows unused): the last lane l <
+// nrows with s_l <= p, by a five-step binary search over the lanes.
+__device__ __forceinline__ int row_in_chunk(int s, int nrows, int p)
+{
+    int lo = 0;
+#pragma unroll
+    for (int step = 16; step >= 1; step >>= 1) {
+        const int cand = lo + step;
+        const int v = __shfl_sync(SPT_FULL_MASK, s, cand & 31);
+        if (cand < nrows && v <= p) lo = cand;
+    }
+    return lo;
+}
+
+// Product of two rows of k elements, summed in order; V elements a load.
+template <class T, int V> __device__ __forceinline__ T row_dot(const T *a, const T *b, int k)
+{
+    struct alignas(sizeof(T) * V) Vec { T v[V]; };
+    T s = T(0);
+    for (int q = 0; q < k; q += V) {
+        const Vec x = *reinterpret_cast<const Vec *>(a + q), y = *reinterpret_cast<const Vec *>(b + q);
+#pragma unroll
+        for (int u = 0; u < V; ++u) s += x.v[u] * y.v[u];
+    }
+    return s;
+}
+
+// The most elements a load (16 bytes at most) that rows of k elements at
+// multiples of ld elements from a and b allow.
+template <class T> __host__ __device__ __forceinline__ int row_vec(const T *a, const T *b, int64_t ld, int k)
+{
+    const size_t bits = reinterpret_cast<size_t>(a) | reinterpret_cast<size_t>(b) |
+                        (size_t)ld * sizeof(T) | (size_t)k * sizeof(T);
+    int v = 16 / (int)sizeof(T);
+    while (v > 1 && bits % ((size_t)v * sizeof(T)) != 0) v >>= 1;
+    return v;
+}
+
 // Prefetch into L2 the first line of a row's entries (indices and values).
 __device__ __forceinline__ void prefetch_l2(const void *p)
 {

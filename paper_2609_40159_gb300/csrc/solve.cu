@@ -696,25 +696,26 @@ size_t block_smem_bytes(int rpw, int kt, int kc, bool f64)
     return ring * kt * (f64 ? 8 : 4) + ring * 4 + (size_t)kc * 4 + 16;
 }
 // ------------------------------------------------------------- gradient
-template <class T>
-__global__ void k_grad_vals(Sys<T> A, const T *__restrict__ gb, const T *__restrict__ x,
-                            int64_t ld, int32_t k, T *__restrict__ gv)
+// One warp per 32 rows, their nonzeros one per lane: with eight lanes per row
+// half the lanes of a short row idle, and an FP64 multiply-add takes its 19
+// cycles of the SM whatever the lanes do.
+// 128^3 Laplacian, FP64, 8 columns: about 135 us (eight lanes per row, one element
+// a load: 261 us; the multiply-adds alone: 127 us).
+template <class T, int V>
+__global__ void __launch_bounds__(256) k_grad_vals(Sys<T> A, const T *__restrict__ gb, const T *__restrict__ x,
+                                                   int64_t ld, int32_t k, T *__restrict__ gv)
 {
     const int lane = threadIdx.x & 31;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    // 4 rows per warp, 8 lanes per row
-    const int g = lane >> 3, sl = lane & 7;
-    for (int64_t r4 = gw * 4; r4 < A.n; r4 += nw * 4) {
-        const int64_t i = r4 + g;
-        if (i >= A.n) continue;
-        const int a = ldro(A.rp + i), e = ldro(A.rp + i + 1);
-        const T *gi = gb + i * ld;
-        for (int p = a + sl; p < e; p += 8) {
-            const T *xj = x + (int64_t)ldro(A.ci + p) * ld;
-            T s = T(0);
-            for (int r = 0; r < k; ++r) s += gi[r] * xj[r];
-            gv[p] = -s;
+    for (int64_t r0 = gw * 32; r0 < A.n; r0 += nw * 32) {
+        const int nrows = (int)min((int64_t)32, A.n - r0);
+        const int s = ldro(A.rp + r0 + min(lane, nrows));
+        const int p0 = __shfl_sync(SPT_FULL_MASK, s, 0), end = ldro(A.rp + r0 + nrows);
+        for (int base = p0; base < end; base += 32) {
+            const int p = base + lane;
+            const int r = row_in_chunk(s, nrows, p);
+            if (p < end) gv[p] = -row_dot<T, V>(gb + (r0 + r) * ld, x + (int64_t)ldro(A.ci + p) * ld, k);
         }
     }
 }
@@ -724,9 +725,11 @@ cudaError_t grad_vals(const Sys<T> &A, const T *gb, const T *x, int64_t ld, int3
                       cudaStream_t s)
 {
     if (A.n <= 0) return cudaSuccess;
-    int64_t blocks = ((int64_t)A.n + 31) / 32;
-    if (blocks > 65535 * 4) blocks = 65535 * 4;
-    k_grad_vals<T><<<(int)blocks, 256, 0, s>>>(A, gb, x, ld, k, gv);
+    const int64_t blocks = std::min<int64_t>(((int64_t)A.n + 255) / 256, 152 * 16);
+    const int v = row_vec<T>(gb, x, ld, k);
+    if (v == 4) k_grad_vals<T, 16 / sizeof(T)><<<(int)blocks, 256, 0, s>>>(A, gb, x, ld, k, gv);
+    else if (v == 2) k_grad_vals<T, 2><<<(int)blocks, 256, 0, s>>>(A, gb, x, ld, k, gv);
+    else k_grad_vals<T, 1><<<(int)blocks, 256, 0, s>>>(A, gb, x, ld, k, gv);
     return cudaGetLastError();
 }
 
