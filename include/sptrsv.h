@@ -243,7 +243,8 @@ sptrsv_status sptrsv_solve(sptrsv_plan plan, const void *b, void *x, int32_t nrh
 /* Adjoint of the solve: g_b = L^{-T} g_x, processed in reverse level /
  * reverse row order.  Requires build_transpose.  Asynchronous.  L's current
  * values are read on every call (most schedules first gather them into CSC
- * order in a plan-owned buffer), so values may change between calls.      */
+ * order in a plan-owned buffer), so values may change between calls.  gx and
+ * gb must not overlap.                                                     */
 sptrsv_status sptrsv_solve_transpose(sptrsv_plan plan, const void *gx, void *gb, int32_t nrhs,
                                      int64_t ld);
 
@@ -342,7 +343,8 @@ sptrsv_status sptrsv_batch_plan_set_schedule(sptrsv_plan plan, int32_t direction
                                              const int32_t *schedule);
 /* All systems in one persistent launch (plus a tiny reset launch and one
  * that lays the current values out for it): no host work per matrix, so the
- * call can be captured in a CUDA graph.                                    */
+ * call can be captured in a CUDA graph.  x may be b itself (the right-hand
+ * sides are then copied to a temporary buffer of the stream's pool first).  */
 sptrsv_status sptrsv_batch_solve(sptrsv_plan plan, const void *b, void *x);
 sptrsv_status sptrsv_batch_solve_transpose(sptrsv_plan plan, const void *gx, void *gb);
 sptrsv_status sptrsv_batch_grad_vals(sptrsv_plan plan, const void *gb, const void *x,

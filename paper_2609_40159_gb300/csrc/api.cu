@@ -166,6 +166,7 @@ struct sptrsv_plan_st {
     struct Geom {
         std::vector<int32_t> rpw, tile, sched;
         bool csc_vals = false;  // some item reads L's values in CSC order
+        bool strips = false;    // some item is solved over strips
         BatchItem *d_items = nullptr;
         int32_t *d_order = nullptr;
         int32_t nitems = 0;
@@ -684,6 +685,44 @@ int auto_mode(const PlanMat &M)
     return SPTRSV_MODE_HYBRID;
 }
 
+// Whether two [n x k] blocks of one leading dimension (elements of w bytes)
+// share an element: their spans meet, and x is not made of other columns of
+// b's rows.
+bool share_elements(const void *b, const void *x, int32_t n, int32_t k, int64_t ld, size_t w)
+{
+    const int64_t span = ((int64_t)(n - 1) * ld + k) * (int64_t)w;
+    const int64_t d = (const char *)x - (const char *)b;
+    if (d >= span || -d >= span) return false;
+    const int64_t row = ld * (int64_t)w, width = k * (int64_t)w;
+    const int64_t at = ((d % row) + row) % row;  // x's first column, from the start of a row of b
+    return at < width || at + width > row;
+}
+
+// The solves over strips read b a second time where a solution is not finite
+// (strip.cuh), after x has been written: where the two share elements they
+// read this copy of b, which has the same leading dimension.
+struct OwnRhs {
+    void *copy = nullptr;
+    cudaStream_t s = nullptr;
+    cudaError_t take(const void **b, int64_t n, int64_t k, int64_t ld, size_t w, cudaStream_t stream)
+    {
+        s = stream;
+        const size_t span = ((size_t)(n - 1) * (size_t)ld + (size_t)k) * w, row = (size_t)ld * w;
+        cudaError_t e = cudaMallocAsync(&copy, span, s);
+        if (e != cudaSuccess) { copy = nullptr; return e; }
+        if (n == 1 || k == ld)
+            e = cudaMemcpyAsync(copy, *b, span, cudaMemcpyDeviceToDevice, s);
+        else
+            e = cudaMemcpy2DAsync(copy, row, *b, row, (size_t)k * w, (size_t)n, cudaMemcpyDeviceToDevice, s);
+        *b = copy;
+        return e;
+    }
+    ~OwnRhs()
+    {
+        if (copy) cudaFreeAsync(copy, s);
+    }
+};
+
 template <class T>
 sptrsv_status solve_impl(sptrsv_plan p, const void *b, void *x, int32_t nrhs, int64_t ld, bool trans)
 {
@@ -693,13 +732,18 @@ sptrsv_status solve_impl(sptrsv_plan p, const void *b, void *x, int32_t nrhs, in
     if (trans && !p->have_csc) return SPTRSV_ENOTSUP;
     cudaStream_t s = p->h->stream;
     Sys<T> A = sys_of<T>(M, p->h->d_status);
-    Rhs<T> R{(const T *)b, (T *)x, ld, nrhs};
     int mode = p->mode;
     if (mode == SPTRSV_MODE_BLOCK && !block_mode_supported(nrhs, sizeof(T) == 8)) mode = SPTRSV_MODE_SYNCFREE;
     const int dir = trans ? 1 : 0;
     // schedules that lay the values out themselves
     const bool strips = mode == SPTRSV_MODE_BLOCK && p->rpw == 32 && M.strips[dir].blocks != nullptr;
     const bool flow = mode == SPTRSV_MODE_HYBRID && use_flow(p, dir);
+    OwnRhs own;
+    if (strips && share_elements(b, x, M.L.n, nrhs, ld, sizeof(T))) {
+        cudaError_t eo = own.take(&b, M.L.n, nrhs, ld, sizeof(T), s);
+        if (eo != cudaSuccess) return from_cuda(eo);
+    }
+    Rhs<T> R{(const T *)b, (T *)x, ld, nrhs};
     // (k_level_cols fills x before it reads b)
     const size_t span = ((size_t)(M.L.n - 1) * (size_t)ld + (size_t)nrhs) * sizeof(T);
     const bool apart = (const char *)b + span <= (const char *)x || (const char *)x + span <= (const char *)b;
@@ -1124,7 +1168,7 @@ sptrsv_status rebuild_items(sptrsv_plan p, int dir)
     std::vector<BatchItem> items;
     std::vector<double> est;
     size_t smem = 16;
-    G.csc_vals = false;
+    G.csc_vals = G.strips = false;
     auto takes_strips = [&](int m) { return G.rpw[m] == 32 && G.sched[m] == kSchedInOrder && p->mats[m].L.n > 0; };
     std::vector<PlanMat *> need;
     if (dir == 0 || p->have_csc)
@@ -1155,6 +1199,7 @@ sptrsv_status rebuild_items(sptrsv_plan p, int dir)
             I.sched = G.sched[m];
             I.rpw = I.sched == kSchedLevel ? 32 : G.rpw[m] == 32 && !one_lane ? 16 : G.rpw[m];
             if (I.sched == kSchedInOrder && I.rpw == 32) {
+                G.strips = true;
                 I.nw = kBatchWarps;
                 smem = std::max(smem, strip_smem(M.strips[dir].ring, I.KT, f64, kBatchWarps));
             } else {
@@ -1466,6 +1511,13 @@ sptrsv_status batch_solve_impl(sptrsv_plan p, const void *b, void *x, bool trans
     if (!b || !x) return SPTRSV_EINVAL;
     if (trans && !p->have_csc) return SPTRSV_ENOTSUP;
     p->last_dir = trans ? 1 : 0;
+    OwnRhs own;
+    const int64_t total = p->rhs_off.back();
+    const size_t wb = p->dtype == SPTRSV_F64 ? 8 : 4;
+    if (G.strips && (const char *)x < (const char *)b + total * wb && (const char *)b < (const char *)x + total * wb) {
+        cudaError_t eo = own.take(&b, 1, total, total, wb, p->h->stream);
+        if (eo != cudaSuccess) return from_cuda(eo);
+    }
     Waiter w{p->h->d_status, &p->d_ctl->abort_flag, p->spin};
     cudaError_t e = cudaSuccess;
     if (trans && G.csc_vals)
