@@ -522,15 +522,18 @@ int flow_grid(int64_t work) { return (int)std::min<int64_t>(std::max<int64_t>((w
 
 template <class T, bool TR> cudaError_t flow_config(cudaLaunchConfig_t &c, cudaLaunchAttribute *at, int csize)
 {
-    static bool done = false;  // one flag per kernel instantiation
+    static DeviceOnce once;  // one per kernel instantiation
     constexpr int smem = Ring<T>::R * Ring<T>::kBytes + 16;  // the ring and the slot that is always ready
-    if (!done) {
-        cudaError_t e = cudaFuncSetAttribute(k_flow<T, TR>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_flow<T, TR>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return e;
-        done = true;
-    }
+    int device = -1;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e == cudaSuccess)
+        e = (cudaError_t)once.run(device, [] {
+            cudaError_t q = cudaFuncSetAttribute(k_flow<T, TR>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (q == cudaSuccess)
+                q = cudaFuncSetAttribute(k_flow<T, TR>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            return (int)q;
+        });
+    if (e != cudaSuccess) return e;
     c.blockDim = dim3(kFlowThreads);
     c.dynamicSmemBytes = smem;
     at[0].id = cudaLaunchAttributeClusterDimension;

@@ -938,17 +938,6 @@ int block_warps_for(double rows_per_level, int rpw)
     return w;
 }
 
-// The dynamic shared-memory limit is raised once per kernel instantiation
-// (outside any stream capture: plans run a first solve before capturing).
-template <auto Kernel> static void raise_smem_once()
-{
-    static bool done = false;  // one flag per kernel instantiation
-    if (!done) {
-        cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBlockSmemBudget);
-        done = true;
-    }
-}
-
 template <class T, int KT>
 static cudaError_t blk_launch(const Sys<T> &A, const Rhs<T> &R, int rpw, bool trans,
                               const SyncArgs &sy, int nwarps, cudaStream_t s)
@@ -958,11 +947,12 @@ static cudaError_t blk_launch(const Sys<T> &A, const Rhs<T> &R, int rpw, bool tr
     const size_t smem = block_smem_bytes(rpw, KT, kc, sizeof(T) == 8);
     if (smem > kBlockSmemBudget) return cudaErrorInvalidConfiguration;
     const int tiles = (R.k + KT - 1) / KT;
+    const cudaError_t e = trans ? allow_smem<k_block<T, KT, true>>((int)kBlockSmemBudget)
+                                : allow_smem<k_block<T, KT, false>>((int)kBlockSmemBudget);
+    if (e != cudaSuccess) return e;
     if (trans) {
-        raise_smem_once<k_block<T, KT, true>>();
         k_block<T, KT, true><<<tiles, kBlockThreads, smem, s>>>(A, R, rpw, kc, P, nwarps, sy);
     } else {
-        raise_smem_once<k_block<T, KT, false>>();
         k_block<T, KT, false><<<tiles, kBlockThreads, smem, s>>>(A, R, rpw, kc, P, nwarps, sy);
     }
     return cudaGetLastError();
@@ -975,11 +965,12 @@ static cudaError_t strip_launch(const Sys<T> &A, const Strips &V, const Rhs<T> &
     const size_t smem = strip_smem(V.ring, KT, sizeof(T) == 8, kStripWarps);
     if (smem > kBlockSmemBudget) return cudaErrorInvalidConfiguration;
     const int tiles = (R.k + KT - 1) / KT;
+    const cudaError_t e = trans ? allow_smem<k_strip<T, KT, true>>((int)kBlockSmemBudget)
+                                : allow_smem<k_strip<T, KT, false>>((int)kBlockSmemBudget);
+    if (e != cudaSuccess) return e;
     if (trans) {
-        raise_smem_once<k_strip<T, KT, true>>();
         k_strip<T, KT, true><<<tiles, 32 * kStripWarps, smem, s>>>(A, V, R, sy);
     } else {
-        raise_smem_once<k_strip<T, KT, false>>();
         k_strip<T, KT, false><<<tiles, 32 * kStripWarps, smem, s>>>(A, V, R, sy);
     }
     return cudaGetLastError();

@@ -3,6 +3,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "device_once.h"
 #include "internal.h"
 
 namespace spt {
@@ -88,6 +89,18 @@ struct Strips {
 };
 
 // ---------------------------------------------------------------- launchers
+// Raises the dynamic shared memory that a kernel may take on the current
+// device, once per device.
+template <auto Kernel> cudaError_t allow_smem(int bytes)
+{
+    static DeviceOnce once;  // one per kernel instantiation
+    int device = -1;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    return (cudaError_t)once.run(
+        device, [&] { return (int)cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
+}
+
 // All return cudaSuccess or the launch error; T = double or float.
 template <class T>
 cudaError_t launch_prologue(PlanCtl *ctl, cudaStream_t s);

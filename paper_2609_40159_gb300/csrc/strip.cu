@@ -371,16 +371,6 @@ int stage_grid(int64_t groups)
     return (int)std::min<int64_t>(std::max<int64_t>((groups + kStageWarps - 1) / kStageWarps, 1), 152 * 8);
 }
 
-// (outside any capture: plans stage once before they are captured)
-template <auto Kernel> void allow_smem(int bytes)
-{
-    static bool done = false;  // one flag per kernel instantiation
-    if (!done) {
-        cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        done = true;
-    }
-}
-
 }  // namespace
 
 cudaError_t strip_sizes(const StripBuild &B, cudaStream_t s)
@@ -405,13 +395,10 @@ template <class T> cudaError_t strip_stage(const Sys<T> &A, const Strips &V, boo
     if (A.n <= 0) return cudaSuccess;
     constexpr int smem = kStageWarps * kStageBytes<T>;
     const int grid = stage_grid(((int64_t)A.n + 31) / 32);
-    if (trans) {
-        allow_smem<k_strip_stage<T, true>>(smem);
-        k_strip_stage<T, true><<<grid, 32 * kStageWarps, smem, s>>>(A, V);
-    } else {
-        allow_smem<k_strip_stage<T, false>>(smem);
-        k_strip_stage<T, false><<<grid, 32 * kStageWarps, smem, s>>>(A, V);
-    }
+    const cudaError_t e = trans ? allow_smem<k_strip_stage<T, true>>(smem) : allow_smem<k_strip_stage<T, false>>(smem);
+    if (e != cudaSuccess) return e;
+    if (trans) k_strip_stage<T, true><<<grid, 32 * kStageWarps, smem, s>>>(A, V);
+    else k_strip_stage<T, false><<<grid, 32 * kStageWarps, smem, s>>>(A, V);
     return cudaGetLastError();
 }
 
@@ -420,9 +407,10 @@ cudaError_t strip_stage_batch(const BatchMat *mats, const RowChunk *chunks, int6
                               cudaStream_t s)
 {
     constexpr int smem = kStageWarps * kStageBytes<T>;
-    allow_smem<k_strip_stage_batch<T, true>>(smem);
-    allow_smem<k_strip_stage_batch<T, false>>(smem);
-    if (nchunks <= 0) return cudaSuccess;
+    // (both, also without chunks: a plan calls this once outside any capture)
+    cudaError_t e = allow_smem<k_strip_stage_batch<T, true>>(smem);
+    if (e == cudaSuccess) e = allow_smem<k_strip_stage_batch<T, false>>(smem);
+    if (e != cudaSuccess || nchunks <= 0) return e;
     const int grid = stage_grid(nchunks);
     if (trans) k_strip_stage_batch<T, true><<<grid, 32 * kStageWarps, smem, s>>>(mats, chunks, nchunks);
     else k_strip_stage_batch<T, false><<<grid, 32 * kStageWarps, smem, s>>>(mats, chunks, nchunks);
