@@ -129,7 +129,11 @@ __device__ __forceinline__ double ld_x(const double *p)
 constexpr int kFlowThreads = 512;
 constexpr int kFlowWarps = kFlowThreads / 32;
 
-// Waits of one block: gives up once for the whole cluster.
+// Waits of one block.  A warp that gives up tells its cluster (the abort words
+// in shared memory, looked at often) and the other right-hand sides' clusters
+// (the plan's abort flag, read by a block when it starts and every 4,096
+// polls): more clusters than the GPU holds run in waves, which would otherwise
+// wait the whole limit one after another.
 struct FlowWait {
     Waiter w;
     unsigned abort_at;  // shared address of the block's abort word
@@ -146,7 +150,7 @@ struct FlowWait {
     }
     __device__ __forceinline__ void give_up() const
     {
-        set_status(w.status, SPTRSV_ETIMEOUT);
+        spt::give_up(w);
         for (int c = 0; c < csize; ++c)
             asm volatile("st.relaxed.cluster.shared::cluster.s32 [%0], %1;" ::"r"(map_rank(abort_at, c)), "r"(1)
                          : "memory");
@@ -154,7 +158,7 @@ struct FlowWait {
 };
 
 // Bound of a polling loop that a whole warp runs together: false once the
-// wait limit has passed or another warp of the cluster gave up.
+// wait limit has passed or another warp gave up.
 struct FlowClock {
     long long start = 0;
     unsigned polls = 0;
@@ -162,6 +166,7 @@ struct FlowClock {
     {
         if ((++polls & 63u) != 0) return true;
         if (__any_sync(SPT_FULL_MASK, fw.gave_up())) return false;
+        if ((polls & 4095u) == 0 && __any_sync(SPT_FULL_MASK, aborted(fw.w))) return false;
         const long long t = clock64();
         if (start == 0) start = t;
         if (__any_sync(SPT_FULL_MASK, (double)(t - start) > 2.2 * (double)fw.w.limit_ns)) {
@@ -236,8 +241,9 @@ __device__ __forceinline__ int meta_most(uint32_t m) { return (m >> 20) & 15; }
 
 // The values in the order that the solve reads them (every solve: L's values
 // may have changed since the last).
-template <class T, bool TR> __global__ void __launch_bounds__(256) k_flow_stage(Sys<T> A, FlowSched F)
+template <class T, bool TR> __global__ void __launch_bounds__(256) k_flow_stage(Sys<T> A, FlowSched F, Waiter w)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) st_relaxed(w.abort_flag, 0);  // for the solve that follows
     const int64_t nslots = (int64_t)F.ngroups * 32;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nslots; t += (int64_t)gridDim.x * blockDim.x) {
         const FlowLane ln = F.lanes[t];
@@ -270,7 +276,7 @@ k_flow(Sys<T> A, FlowSched F, Rhs<T> R, int32_t withhold, Waiter w)
     const unsigned ring = smem_addr(smraw);
     for (int t = threadIdx.x; t < NR * SB / 16 + 1; t += kFlowThreads)
         reinterpret_cast<uint4 *>(smraw)[t] = make_uint4(0u, 0u, 0u, 0u);
-    if (threadIdx.x == 0) s_abort = 0;
+    if (threadIdx.x == 0) s_abort = aborted(w) ? 1 : 0;
     const FlowWait fw{w, smem_addr(&s_abort), F.csize};
     cluster_arrive();
     const int nepochs = (F.n + H - 1) / H;
@@ -403,15 +409,14 @@ k_flow(Sys<T> A, FlowSched F, Rhs<T> R, int32_t withhold, Waiter w)
             }
             for (int o = lpr >> 1; o > 0; o >>= 1) acc += shfl_xor(acc, o);
         }
+        if (!ok) break;  // (what is left are the barriers, which the other warps count on)
         const T xi = (bv - acc) * rinv;
-        if (ok) {
-            if (anythere) {
-                if (there) slot_store<true>(other, xi, me.code);
-                if (anymore)
-                    for (unsigned m = mask; m; m &= m - 1) slot_store<true>(map_rank(own, __ffs(m) - 1), xi, me.code);
-            }
-            if (here) slot_store<false>(own, xi, me.code);
+        if (anythere) {
+            if (there) slot_store<true>(other, xi, me.code);
+            if (anymore)
+                for (unsigned m = mask; m; m &= m - 1) slot_store<true>(map_rank(own, __ffs(m) - 1), xi, me.code);
         }
+        if (here) slot_store<false>(own, xi, me.code);
         if (lead) x[(int64_t)me.row * R.ld] = xi;
         __syncwarp();
     }
@@ -608,8 +613,8 @@ cudaError_t solve_flow(const Sys<T> &A, const FlowSched &F, const Rhs<T> &R, boo
     c.gridDim = dim3((unsigned)(F.csize * R.k));
     c.stream = s;
     const int sg = flow_grid((int64_t)F.ngroups * 32);
-    if (trans) k_flow_stage<T, true><<<sg, 256, 0, s>>>(A, F);
-    else k_flow_stage<T, false><<<sg, 256, 0, s>>>(A, F);
+    if (trans) k_flow_stage<T, true><<<sg, 256, 0, s>>>(A, F, w);
+    else k_flow_stage<T, false><<<sg, 256, 0, s>>>(A, F, w);
     return trans ? cudaLaunchKernelEx(&c, k_flow<T, true>, A, F, R, withhold, w)
                  : cudaLaunchKernelEx(&c, k_flow<T, false>, A, F, R, withhold, w);
 }

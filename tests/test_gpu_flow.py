@@ -104,3 +104,34 @@ def test_flow_bounded_wait(trans):
     ref = (oracle.solve_transpose if trans else oracle.solve)(A_h, b_h)
     assert relerr(run(b).cpu().numpy(), ref) <= 1e-12
     assert h.status() == 0
+
+
+@pytest.mark.parametrize("trans", [False, True], ids=["fwd", "transpose"])
+def test_flow_gives_up_once_for_all_columns(trans):
+    """One cluster per right-hand side, more of them than the GPU holds at a
+    time (one block on an SM): a row that never comes ends the solve after
+    about one wait limit, not after one for every wave of clusters."""
+    import time
+
+    import paper_2609_40159_gb300 as P
+    A_h = S.lap2d(200)
+    k = 4 * torch.cuda.get_device_properties(0).multi_processor_count  # four waves at least
+    limit_s = 0.4
+    b_h = S.rhs(A_h.n, k, seed=2, dtype=np.float32)
+    b = torch.as_tensor(b_h).cuda()
+    plan = P.Plan(P.Matrix.from_host(A_h.astype(np.float32)), mode="hybrid", transpose=True,
+                  wait_limit_us=int(1e6 * limit_s))
+    h = P.handle()
+    run = plan.solve_transpose if trans else plan.solve
+    run(b)
+    torch.cuda.synchronize()
+    plan.withhold(200 * 100 + 100)
+    t0 = time.perf_counter()
+    run(b)
+    assert h.status() == P._lib.SPTRSV_ETIMEOUT
+    # (the limit is counted at 2.2 GHz, above the clock: up to half as long again)
+    assert time.perf_counter() - t0 < 2.5 * limit_s
+    plan.withhold(-1)
+    ref = (oracle.solve_transpose if trans else oracle.solve)(A_h, b_h[:, -3:].astype(np.float64))
+    assert relerr(run(b).cpu().numpy()[:, -3:], ref) <= TOL[np.float32]
+    assert h.status() == 0
