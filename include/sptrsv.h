@@ -298,7 +298,7 @@ sptrsv_status sptrsv_plan_set_thin_rows(sptrsv_plan plan, int32_t thin_rows);
  * otherwise at most that many.  Their waiting warps poll global memory, so
  * fewer of them can be faster.  Any value is correct: a row group only
  * waits on groups taken before it.  Returns SPTRSV_EINVAL for a negative
- * value or a batched plan.                                                */
+ * value or a batched plan.  Builds whatever schedule data the setting needs.  */
 sptrsv_status sptrsv_plan_set_blocks_per_sm(sptrsv_plan plan, int32_t blocks_per_sm);
 
 /* Re-tunes a batched plan (used by the autotuner; no analysis is repeated).
@@ -441,6 +441,13 @@ sptrsv_status sptrsv_debug_withhold_row(sptrsv_plan plan, int32_t row);
  * published, every wait of those calls gives up after wait_limit_us (> 0)
  * and they return SPTRSV_ETIMEOUT; row = -1 clears the hook.               */
 sptrsv_status sptrsv_debug_withhold_level(sptrsv_handle handle, int32_t row, int64_t wait_limit_us);
+
+/* Test hook for plans that get no memory for a schedule's tables (the cluster
+ * flow of the hybrid mode, the strips of the block mode and of batches): the
+ * plans that `handle` makes or changes from now on take tables of more than
+ * `bytes` for an allocation that failed and solve without them; -1 clears
+ * the hook.                                                                 */
+sptrsv_status sptrsv_debug_limit_tables(sptrsv_handle handle, int64_t bytes);
 
 #ifdef __cplusplus
 }

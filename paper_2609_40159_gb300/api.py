@@ -82,6 +82,11 @@ class Handle:
         L.check(L.lib().sptrsv_debug_withhold_level(self.h, int(row), int(wait_limit_us)),
                 "sptrsv_debug_withhold_level")
 
+    def limit_tables(self, nbytes: int = -1):
+        """Test hook: schedule tables of more than nbytes count as an
+        allocation that failed (see sptrsv_debug_limit_tables); -1 clears it."""
+        L.check(L.lib().sptrsv_debug_limit_tables(self.h, int(nbytes)), "sptrsv_debug_limit_tables")
+
     def __del__(self):
         try:
             if getattr(self, "h", None) and not L.exiting():

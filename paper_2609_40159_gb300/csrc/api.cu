@@ -97,6 +97,7 @@ struct sptrsv_handle_st {
     // test hook of the level analysis (sptrsv_debug_withhold_level)
     int32_t dbg_withhold = -1;
     long long dbg_wait_ns = 0;
+    int64_t dbg_table_limit = -1;  // (sptrsv_debug_limit_tables)
 };
 
 struct PlanMat {
@@ -150,7 +151,7 @@ struct sptrsv_plan_st {
     // cluster flow schedule of each direction ([0] forward, [1] transpose),
     // built when the hybrid mode is chosen; off: could not be built
     FlowSched flow[2];
-    bool flow_ready[2] = {false, false}, flow_off = false;
+    bool flow_ready[2] = {false, false}, flow_off[2] = {false, false};
     // row-major copies of a column-major right-hand-side block and its
     // solution (sptrsv_solve_layout), grown on demand
     void *d_lay = nullptr;
@@ -200,6 +201,17 @@ struct sptrsv_plan_st {
         cudaError_t e = cudaMalloc(&q, bytes > 0 ? bytes : 16);
         if (e == cudaSuccess) { owned.push_back(q); *p = static_cast<P *>(q); }
         return e;
+    }
+    // Tables of a schedule that the plan can do without.
+    template <class P> cudaError_t alloc_tables(P **p, size_t bytes)
+    {
+        if (h->dbg_table_limit >= 0 && bytes > (size_t)h->dbg_table_limit) return cudaErrorMemoryAllocation;
+        return alloc(p, bytes);
+    }
+    void release(void *q)
+    {
+        owned.erase(std::remove(owned.begin(), owned.end(), q), owned.end());
+        cudaFree(q);
     }
 };
 
@@ -538,13 +550,14 @@ void build_strips(sptrsv_plan p, const std::vector<PlanMat *> &mats, int dir)
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e == cudaSuccess && total > INT32_MAX) e = cudaErrorMemoryAllocation;  // (32 GB)
     const size_t b_blocks = 16 * (size_t)total;
-    if (e == cudaSuccess) e = p->alloc(&tab, b_blocks + b_ofs + 2 * (size_t)nnz);
+    if (e == cudaSuccess) e = p->alloc_tables(&tab, b_blocks + b_ofs + 2 * (size_t)nnz);
     if (e == cudaSuccess) {
         uint32_t *ofs = reinterpret_cast<uint32_t *>(tab + b_blocks);
         uint16_t *ecode = reinterpret_cast<uint16_t *>(tab + b_blocks + b_ofs);
         e = cudaMemcpyAsync(ofs, B.ofs, b_ofs, cudaMemcpyDeviceToDevice, s);
         if (e == cudaSuccess) e = strip_tables(B, ofs, reinterpret_cast<unsigned char *>(tab), ecode, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) p->release(tab);
         for (size_t m = 0; m < nm && e == cudaSuccess; ++m)
             mats[m]->strips[dir] = Strips{reinterpret_cast<unsigned char *>(tab), ofs + src[m].g0, ecode + src[m].e0,
                                           strip_ring(far[m], B.ring_most)};
@@ -608,21 +621,22 @@ sptrsv_status build_flow(sptrsv_plan p, int dir)
         all.insert(all.end(), v.begin(), v.end());
         gptr.push_back((int32_t)all.size());
     }
+    // one allocation, so that nothing is left of tables that cannot be had
     const size_t ns = 32 * std::max<size_t>(all.size(), 1), w = f64 ? 8 : 4;
-    FlowLane *lanes = nullptr;
-    uint4 *codes = nullptr;
-    int2 *src = nullptr;
-    uint32_t *ecode = nullptr;
+    const size_t at_codes = sizeof(FlowLane) * ns, at_vals = at_codes + sizeof(uint4) * ns;
+    const size_t at_inv = at_vals + 4 * w * ns, at_src = at_inv + w * ns, at_ecode = at_src + sizeof(int2) * ns;
+    const size_t at_gptr = at_ecode + sizeof(uint32_t) * (size_t)M.L.nnz;
+    char *tab = nullptr;
     FlowGroup *groups = nullptr;
-    int32_t *d_gptr = nullptr;
+    if (e == cudaSuccess) e = p->alloc_tables(&tab, at_gptr + sizeof(int32_t) * gptr.size());
+    FlowLane *lanes = reinterpret_cast<FlowLane *>(tab);
+    uint4 *codes = reinterpret_cast<uint4 *>(tab + at_codes);
+    int2 *src = reinterpret_cast<int2 *>(tab + at_src);
+    uint32_t *ecode = reinterpret_cast<uint32_t *>(tab + at_ecode);
+    int32_t *d_gptr = reinterpret_cast<int32_t *>(tab + at_gptr);
     FlowSched F{};
-    if (e == cudaSuccess) e = p->alloc(&lanes, sizeof(FlowLane) * ns);
-    if (e == cudaSuccess) e = p->alloc(&codes, sizeof(uint4) * ns);
-    if (e == cudaSuccess) e = p->alloc(&src, sizeof(int2) * ns);
-    if (e == cudaSuccess) e = p->alloc(&ecode, sizeof(uint32_t) * (size_t)M.L.nnz);
-    if (e == cudaSuccess) e = p->alloc(&F.vals, 4 * w * ns);
-    if (e == cudaSuccess) e = p->alloc(&F.inv, w * ns);
-    if (e == cudaSuccess) e = p->alloc(&d_gptr, sizeof(int32_t) * gptr.size());
+    F.vals = tab + at_vals;
+    F.inv = tab + at_inv;
     if (e == cudaSuccess) e = cudaMallocAsync(&groups, sizeof(FlowGroup) * std::max<size_t>(all.size(), 1), s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(groups, all.data(), sizeof(FlowGroup) * all.size(), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_gptr, gptr.data(), sizeof(int32_t) * gptr.size(), cudaMemcpyHostToDevice, s);
@@ -632,7 +646,10 @@ sptrsv_status build_flow(sptrsv_plan p, int dir)
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     cudaFreeAsync(order, s);
     if (groups) cudaFreeAsync(groups, s);
-    if (e != cudaSuccess) return from_cuda(e);
+    if (e != cudaSuccess) {
+        if (tab) p->release(tab);
+        return from_cuda(e);
+    }
     F.lanes = lanes;
     F.codes = codes;
     F.src = src;
@@ -646,27 +663,28 @@ sptrsv_status build_flow(sptrsv_plan p, int dir)
     return SPTRSV_OK;
 }
 
-// Whether solves of direction dir run the cluster flow schedule: the hybrid
+// Whether the plan's settings call for the cluster flow schedule: the hybrid
 // mode with its automatic threshold (one synchronisation-free run in level
-// order) and grid.  Where the tables cannot be had, the grid-wide hybrid
-// kernel runs.
-bool use_flow(sptrsv_plan p, int dir)
+// order) and grid.
+bool flow_wanted(const sptrsv_plan_st *p)
 {
-    if (p->mode != SPTRSV_MODE_HYBRID || p->thin_rows != 0 || p->flow_off || p->M.L.n == 0) return false;
-    if (p->grid_level != p->grid_level_max) return false;
-    if (p->flow_ready[dir]) return true;
-    if (build_flow(p, dir) != SPTRSV_OK) p->flow_off = true;
-    return !p->flow_off;
+    return p->mode == SPTRSV_MODE_HYBRID && p->thin_rows == 0 && p->grid_level == p->grid_level_max && p->M.L.n > 0;
 }
 
-// Builds the tables of the plan's mode, so that a solve launches kernels only.
-void prepare_schedules(sptrsv_plan p)
+// Builds the tables of the plan's mode and settings, so that a solve launches
+// kernels only: called by whatever changes them.  Where the flow's tables
+// cannot be had, the grid-wide hybrid kernel runs.
+sptrsv_status prepare_schedules(sptrsv_plan p)
 {
+    bool grid_wide = false;
     for (int dir = 0; dir < (p->have_csc ? 2 : 1); ++dir) {
-        use_flow(p, dir);
+        if (flow_wanted(p) && !p->flow_ready[dir] && !p->flow_off[dir])
+            p->flow_off[dir] = build_flow(p, dir) != SPTRSV_OK;
+        grid_wide = grid_wide || !flow_wanted(p) || !p->flow_ready[dir];
         if (p->mode == SPTRSV_MODE_BLOCK && p->rpw == 32 && p->M.L.n > 0 && !p->M.strips[dir].blocks)
             build_strips(p, {&p->M}, dir);
     }
+    return p->mode == SPTRSV_MODE_HYBRID && grid_wide ? ensure_hybrid(p) : SPTRSV_OK;
 }
 
 // Mode from the mean level width: narrow (deep) systems stay on one SM, very
@@ -737,7 +755,7 @@ sptrsv_status solve_impl(sptrsv_plan p, const void *b, void *x, int32_t nrhs, in
     const int dir = trans ? 1 : 0;
     // schedules that lay the values out themselves
     const bool strips = mode == SPTRSV_MODE_BLOCK && p->rpw == 32 && M.strips[dir].blocks != nullptr;
-    const bool flow = mode == SPTRSV_MODE_HYBRID && use_flow(p, dir);
+    const bool flow = flow_wanted(p) && p->flow_ready[dir];
     OwnRhs own;
     if (strips && share_elements(b, x, M.L.n, nrhs, ld, sizeof(T))) {
         cudaError_t eo = own.take(&b, M.L.n, nrhs, ld, sizeof(T), s);
@@ -964,7 +982,7 @@ extern "C" sptrsv_status sptrsv_plan_create(sptrsv_handle h, const sptrsv_csr *L
     st = ensure_chunks(p);
     if (st == SPTRSV_OK) st = from_cuda(cudaStreamSynchronize(h->stream));
     if (st != SPTRSV_OK) { sptrsv_plan_destroy(p); return st; }
-    prepare_schedules(p);
+    prepare_schedules(p);  // (what the solves cannot do without they ask for again)
     *plan = p;
     return SPTRSV_OK;
 }
@@ -991,7 +1009,7 @@ extern "C" sptrsv_status sptrsv_plan_set_thin_rows(sptrsv_plan p, int32_t thin_r
 {
     if (!p || p->batched || thin_rows < 0) return SPTRSV_EINVAL;
     p->thin_rows = thin_rows;
-    return p->mode == SPTRSV_MODE_HYBRID ? ensure_hybrid(p) : SPTRSV_OK;
+    return prepare_schedules(p);
 }
 
 extern "C" sptrsv_status sptrsv_plan_set_blocks_per_sm(sptrsv_plan p, int32_t blocks_per_sm)
@@ -1000,7 +1018,7 @@ extern "C" sptrsv_status sptrsv_plan_set_blocks_per_sm(sptrsv_plan p, int32_t bl
     const int sms = std::max(1, p->h->di.num_sms);
     const int cap = (int)std::min<int64_t>(p->grid_level_max, (int64_t)blocks_per_sm * sms);
     p->grid_level = blocks_per_sm == 0 ? p->grid_level_max : std::max(1, cap);
-    return SPTRSV_OK;
+    return prepare_schedules(p);
 }
 
 extern "C" sptrsv_status sptrsv_plan_info(sptrsv_plan p, int32_t *nlevels, int32_t *mode,
@@ -1141,6 +1159,13 @@ extern "C" sptrsv_status sptrsv_debug_withhold_level(sptrsv_handle h, int32_t ro
     if (!h || (row >= 0 && wait_limit_us <= 0)) return SPTRSV_EINVAL;
     h->dbg_withhold = row < 0 ? -1 : row;
     h->dbg_wait_ns = row < 0 ? 0 : wait_limit_us * 1000;
+    return SPTRSV_OK;
+}
+
+extern "C" sptrsv_status sptrsv_debug_limit_tables(sptrsv_handle h, int64_t bytes)
+{
+    if (!h) return SPTRSV_EINVAL;
+    h->dbg_table_limit = bytes < 0 ? -1 : bytes;
     return SPTRSV_OK;
 }
 
