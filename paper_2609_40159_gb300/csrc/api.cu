@@ -1199,9 +1199,17 @@ sptrsv_status rebuild_items(sptrsv_plan p, int dir)
     if (dir == 0 || p->have_csc)
         for (int m = 0; m < nmat; ++m)
             if (takes_strips(m) && !p->mats[m].strips[dir].blocks) need.push_back(&p->mats[m]);
-    if (!need.empty()) {
-        build_strips(p, need, dir);
-        for (int m = 0; m < nmat; ++m) p->h_mats[m].strips[dir] = p->mats[m].strips[dir];
+    if (!need.empty()) build_strips(p, need, dir);
+    // (only systems solved over them: the others' values need not be laid out
+    // before every solve)
+    bool changed = false;
+    for (int m = 0; m < nmat; ++m) {
+        Strips &V = p->h_mats[m].strips[dir];
+        const Strips use = takes_strips(m) ? p->mats[m].strips[dir] : Strips{};
+        changed = changed || V.blocks != use.blocks;
+        V = use;
+    }
+    if (changed) {
         cudaError_t e = cudaStreamSynchronize(p->h->stream);
         if (e == cudaSuccess)
             e = cudaMemcpy(p->d_mats, p->h_mats.data(), sizeof(BatchMat) * nmat, cudaMemcpyHostToDevice);
@@ -1548,7 +1556,7 @@ sptrsv_status batch_solve_impl(sptrsv_plan p, const void *b, void *x, bool trans
     if (trans && G.csc_vals)
         e = p->dtype == SPTRSV_F64 ? batch_csc_values<double>(p->d_mats, p->d_ctiles, p->n_ctiles, p->h->stream)
                                    : batch_csc_values<float>(p->d_mats, p->d_ctiles, p->n_ctiles, p->h->stream);
-    if (e == cudaSuccess)
+    if (e == cudaSuccess && G.strips)
         e = p->dtype == SPTRSV_F64
                 ? strip_stage_batch<double>(p->d_mats, p->d_gchunks, p->n_gchunks, trans, p->h->stream)
                 : strip_stage_batch<float>(p->d_mats, p->d_gchunks, p->n_gchunks, trans, p->h->stream);

@@ -109,3 +109,51 @@ def test_settings_bring_their_tables():
                 else:
                     _first_solves_captured(plan, A_h)
     torch.cuda.synchronize()
+
+
+def _launches(run):
+    """Number of nodes of run() under capture."""
+    import ctypes
+    with open("/proc/self/maps") as f:
+        path = next(ln.split()[-1] for ln in f if "libcudart.so" in ln)
+    rt = ctypes.CDLL(path)
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g, stream=torch.cuda.current_stream()):
+        run()
+    count = ctypes.c_size_t(0)
+    assert rt.cudaGraphGetNodes(ctypes.c_void_p(g.raw_cuda_graph()), None, ctypes.byref(count)) == 0
+    return count.value
+
+
+def test_batch_lays_out_what_it_reads():
+    """The launch that lays the values out in strips is there only while some
+    system of the direction is solved over them, and a system comes back to
+    them."""
+    import paper_2609_40159_gb300 as P
+    hosts = [S.band_random(n, 60, 0, 6, seed=n) for n in (33, 700, 2100)]
+    ks, nmat = [1, 5, 2], 3
+    bs = [S.rhs(A.n, k, seed=k) for A, k in zip(hosts, ks)]
+    with torch.cuda.stream(torch.cuda.Stream()):
+        plan = P.BatchPlan([P.Matrix.from_host(A) for A in hosts], nrhs=ks, transpose=True)
+        b = torch.as_tensor(np.concatenate([v.reshape(-1) for v in bs])).cuda()
+        out = torch.empty_like(b)
+
+        def check():
+            for run, ref in ((plan.solve, oracle.solve), (plan.solve_transpose, oracle.solve_transpose)):
+                x = run(b)
+                for m, (A, bh) in enumerate(zip(hosts, bs)):
+                    assert relerr(plan.unpack(x, m).cpu().numpy(), ref(A, bh)) <= 1e-12
+            return _launches(lambda: plan.solve(b, out=out)), _launches(lambda: plan.solve_transpose(b, out=out))
+
+        strips = check()
+        plan.set_schedule(["level"] * nmat)
+        # (the transpose: L's values in CSC order instead)
+        assert check() == (strips[0] - 1, strips[1])
+        plan.set_schedule(["inorder"] * nmat)
+        assert check() == strips
+        plan.set_geometry([16] * nmat, direction="forward")
+        assert check() == (strips[0] - 1, strips[1])
+        plan.set_geometry([16, 32, 16], direction="forward")
+        assert check() == strips
+        assert P.handle().status() == 0
+    torch.cuda.synchronize()
