@@ -2,14 +2,19 @@
 
 For a single-system plan it times every candidate (mode, rows per warp, rhs
 tile) with CUDA events and keeps the fastest (winners are cached in a JSON
-file keyed by size class: ``SPTRSV_TUNE_CACHE`` or
-``~/.cache/sptrsv_gb300/tune.json``).  For a batched plan, whose time is a
+file keyed by size class and by the kernels' sources, as a mode's fastest
+setting is that of the kernels it ran: ``SPTRSV_TUNE_CACHE`` or
+``~/.cache/sptrsv_gb300/tune.json``).  Some settings share a kernel (the
+automatic hybrid schedule ignores rows per warp and tile, the block mode with
+32 rows per warp the tile): their times differ by noise alone.  For a batched plan, whose time is a
 makespan, it first sets one right-hand-side tile for every system, then
 refines rows per warp and tile per size class (bucketed average row length
 and number of right-hand sides) by coordinate descent.
 """
 from __future__ import annotations
 
+import functools
+import hashlib
 import json
 import math
 import os
@@ -50,6 +55,17 @@ def _store_cache(c):
         pass
 
 
+@functools.lru_cache(maxsize=None)
+def kernel_version() -> str:
+    """Short hash of the library's sources."""
+    d = os.path.join(os.path.dirname(os.path.abspath(__file__)), "csrc")
+    h = hashlib.sha256()
+    for name in sorted(os.listdir(d)):
+        with open(os.path.join(d, name), "rb") as f:
+            h.update(name.encode() + b"\0" + f.read())
+    return h.hexdigest()[:12]
+
+
 def _bucket(v):
     return int(round(math.log2(max(v, 1e-9)))) if v > 0 else -99
 
@@ -83,9 +99,10 @@ def tune_plan(plan: Plan, b: torch.Tensor, modes=CANDIDATE_MODES, rpws=CANDIDATE
     n, k = plan.A.n, (b.shape[1] if b.dim() == 2 else 1)
     info = plan.info()
     key = size_class(n, plan.A.nnz, info["nlevels"], k, plan.A.dtype)
+    entry = f"{key}:v{kernel_version()}" if use_cache else key
     cache = _load_cache() if use_cache else {}
-    if key in cache:
-        c = cache[key]
+    if entry in cache:
+        c = cache[entry]
         plan.set(c["mode"], c["rows_per_warp"], c["rhs_tile"])
         return dict(key=key, best=c, cached=True, table=[])
     if kts is None:
@@ -103,7 +120,7 @@ def tune_plan(plan: Plan, b: torch.Tensor, modes=CANDIDATE_MODES, rpws=CANDIDATE
     plan.set(best["mode"], best["rows_per_warp"], best["rhs_tile"])
     if use_cache:
         cache = _load_cache()
-        cache[key] = best
+        cache[entry] = best
         _store_cache(cache)
     return dict(key=key, best=best, cached=False, table=table)
 
