@@ -134,7 +134,7 @@ def kernel_source_hash():
     import hashlib
     import re
     h = hashlib.sha256()
-    for fn in ("block.cuh", "strip.cuh", "strip.cu", "batch.cu", "rows.cuh", "common.cuh"):
+    for fn in ("block.cuh", "strip.cuh", "strip.cu", "batch.cu", "rows.cuh", "common.cuh", "solve.cuh"):
         with open(os.path.join(ROOT, "paper_2609_40159_gb300", "csrc", fn)) as fh:
             text = fh.read()
         text = re.sub(r"/\*.*?\*/", "", text, flags=re.S)
