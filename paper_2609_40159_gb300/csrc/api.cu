@@ -19,6 +19,13 @@ using namespace spt;
 
 namespace {
 
+// Device memory for the length of a call.
+template <class T> struct DeviceArray {
+    T *p = nullptr;
+    cudaError_t get(size_t count) { return cudaMalloc(&p, sizeof(T) * count); }
+    ~DeviceArray() { cudaFree(p); }
+};
+
 // Named NVTX range for a profiler timeline (no cost without a tool attached).
 struct Range {
     explicit Range(const char *name) { nvtxRangePushA(name); }
@@ -175,6 +182,16 @@ struct sptrsv_plan_st {
         int grid = 0;
     } geo[2];
     int32_t max_items = 0;
+    bool takes_strips(int d, size_t m) const
+    {
+        return geo[d].rpw[m] == 32 && geo[d].sched[m] == kSchedInOrder && mats[m].L.n > 0;
+    }
+    void strips_to_build(int d, std::vector<PlanMat *> *need)
+    {
+        if (d == 1 && !have_csc) return;
+        for (size_t m = 0; m < mats.size(); ++m)
+            if (takes_strips(d, m) && !mats[m].strips[d].blocks) need->push_back(&mats[m]);
+    }
     int last_dir = 0;  // direction of the last batched solve (for the trace)
     RowChunk *d_gchunks = nullptr, *d_tchunks = nullptr;  // all 32-row chunks; chunks with T rows
     int64_t n_gchunks = 0, n_tchunks = 0;
@@ -195,8 +212,24 @@ struct sptrsv_plan_st {
     cudaStream_t s_h2d = nullptr, s_d2h = nullptr;
     int64_t nsteps = 0;
 
+    // One allocation that the plan's arrays of known size are carved from (one
+    // of more than 1 MB takes 50 us, and 36 us to give back).
+    char *arena = nullptr;
+    size_t arena_left = 0;
+    static size_t padded(size_t bytes) { return (std::max<size_t>(bytes, 1) + 255) / 256 * 256; }
+    void reserve(size_t bytes)
+    {
+        if (alloc(&arena, bytes) == cudaSuccess) arena_left = bytes;
+        else cudaGetLastError();  // (then one by one)
+    }
     template <class P> cudaError_t alloc(P **p, size_t bytes)
     {
+        if (padded(bytes) <= arena_left) {
+            *p = reinterpret_cast<P *>(arena);
+            arena += padded(bytes);
+            arena_left -= padded(bytes);
+            return cudaSuccess;
+        }
         void *q = nullptr;
         cudaError_t e = cudaMalloc(&q, bytes > 0 ? bytes : 16);
         if (e == cudaSuccess) { owned.push_back(q); *p = static_cast<P *>(q); }
@@ -206,7 +239,10 @@ struct sptrsv_plan_st {
     template <class P> cudaError_t alloc_tables(P **p, size_t bytes)
     {
         if (h->dbg_table_limit >= 0 && bytes > (size_t)h->dbg_table_limit) return cudaErrorMemoryAllocation;
-        return alloc(p, bytes);
+        void *q = nullptr;  // (not of the arena: it may be released)
+        cudaError_t e = cudaMalloc(&q, bytes);
+        if (e == cudaSuccess) { owned.push_back(q); *p = static_cast<P *>(q); }
+        return e;
     }
     void release(void *q)
     {
@@ -396,9 +432,21 @@ template <class T> Sys<T> sys_of(const PlanMat &M, int *chk)
     return A;
 }
 
-// Analysis + schedule data + optional CSC for one system of a plan.
+// Bytes of the arrays that prepare_mat allocates.
+size_t mat_bytes(const sptrsv_csr &L, const sptrsv_csr *T, bool want_csc)
+{
+    auto b = [](int64_t count, size_t w) { return sptrsv_plan_st::padded(w * (size_t)std::max<int64_t>(count, 1)); };
+    const int64_t n = std::max(L.n, 1);
+    size_t all = 2 * b(n, 4) + b(n + 1, 4);
+    if (T && T->n > 0) all += 2 * b((n + 31) / 32, 4) + b(n + 1, 4) + 2 * b(T->nnz, 4);
+    if (want_csc) all += b(n + 1, 4) + 2 * b(L.nnz, 4) + b(L.nnz, L.dtype == SPTRSV_F64 ? 8 : 4);
+    return all;
+}
+
+// Analysis + schedule data + optional CSC for one system of a plan; cost:
+// scratch for the level costs (n entries).  The caller synchronises.
 sptrsv_status prepare_mat(sptrsv_plan p, PlanMat &M, const sptrsv_csr &L, const sptrsv_csr *T,
-                          bool want_csc)
+                          bool want_csc, int64_t *cost)
 {
     sptrsv_handle h = p->h;
     cudaStream_t s = h->stream;
@@ -414,11 +462,8 @@ sptrsv_status prepare_mat(sptrsv_plan p, PlanMat &M, const sptrsv_csr &L, const 
     cudaError_t e = p->alloc(&M.d_lev, sizeof(int32_t) * nn);
     if (e == cudaSuccess) e = p->alloc(&M.d_perm, sizeof(int32_t) * nn);
     if (e == cudaSuccess) e = p->alloc(&M.d_level_ptr, sizeof(int32_t) * (nn + 1));
-    int64_t *cost = nullptr;
-    if (e == cudaSuccess) e = cudaMalloc(&cost, sizeof(int64_t) * nn);
-    if (e != cudaSuccess) { cudaFree(cost); return from_cuda(e); }
+    if (e != cudaSuccess) return from_cuda(e);
     sptrsv_status st = analyze_into(h, L, M.d_lev, M.d_perm, M.d_level_ptr, cost, &M.nlevels, nullptr, p->spin);
-    cudaFree(cost);
     if (st != SPTRSV_OK) return st;
     M.h_level_ptr.assign((size_t)M.nlevels + 1, 0);
     if (n > 0) {
@@ -437,7 +482,6 @@ sptrsv_status prepare_mat(sptrsv_plan p, PlanMat &M, const sptrsv_csr &L, const 
             e = M.T.nnz > 0 ? build_csc(M.T.row_ptr, M.T.col_idx, n, M.T.nnz, M.d_tcp, M.d_trow, M.d_ttmap, s)
                             : cudaMemsetAsync(M.d_tcp, 0, sizeof(int32_t) * (nn + 1), s);
         if (e == cudaSuccess) e = build_tmask(M.d_tcp, n, M.d_tcmask, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return from_cuda(e);
     }
     if (want_csc) {
@@ -447,7 +491,6 @@ sptrsv_status prepare_mat(sptrsv_plan p, PlanMat &M, const sptrsv_csr &L, const 
         if (e == cudaSuccess)
             e = p->alloc(&M.d_cv, (L.dtype == SPTRSV_F64 ? 8 : 4) * (size_t)(L.nnz > 0 ? L.nnz : 1));
         if (e == cudaSuccess) e = build_csc(L.row_ptr, L.col_idx, n, L.nnz, M.d_cp, M.d_crow, M.d_tmap, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return from_cuda(e);
     }
     return SPTRSV_OK;
@@ -509,74 +552,96 @@ sptrsv_status ensure_hybrid(sptrsv_plan p)
     return SPTRSV_OK;
 }
 
-// Strips (strip.cuh) of one direction of systems that have none; left out when
-// their memory cannot be had (then the solves take several lanes per row).
-void build_strips(sptrsv_plan p, const std::vector<PlanMat *> &mats, int dir)
+// Strips (strip.cuh) of the systems of each direction that have none; left out
+// when their memory cannot be had (then the solves take several lanes per row).
+// Both directions in one go, as of a small system the allocations (40 us for
+// one from the stream's pool, and as much again when a synchronisation gives
+// it back) and synchronisations are what this takes.  The caller synchronises.
+void build_strips(sptrsv_plan p, const std::vector<PlanMat *> (&mats)[2])
 {
-    if (mats.empty()) return;
-    const size_t nm = mats.size();
-    std::vector<StripSrc> src(nm);
-    int64_t ng = 0, nnz = 0;
-    for (size_t m = 0; m < nm; ++m) {
-        const PlanMat &M = *mats[m];
-        src[m] = StripSrc{dir ? M.d_cp : M.L.row_ptr, dir ? M.d_crow : M.L.col_idx, ng, nnz, M.L.n};
-        ng += ((int64_t)M.L.n + 31) / 32;
-        nnz += M.L.nnz;
-    }
+    const size_t nm[2] = {mats[0].size(), mats[1].size()}, all = nm[0] + nm[1];
+    if (all == 0) return;
+    std::vector<StripSrc> src(all);
+    int64_t ng[2] = {0, 0}, nnz[2] = {0, 0};
+    for (int d = 0; d < 2; ++d)
+        for (size_t m = 0; m < nm[d]; ++m) {
+            const PlanMat &M = *mats[d][m];
+            src[d * nm[0] + m] = StripSrc{d ? M.d_cp : M.L.row_ptr, d ? M.d_crow : M.L.col_idx, ng[d], nnz[d], M.L.n};
+            ng[d] += ((int64_t)M.L.n + 31) / 32;
+            nnz[d] += M.L.nnz;
+        }
     cudaStream_t s = p->h->stream;
+    // scratch: the systems; totals and reaches (read back); then by direction
+    // and group offsets (copied to the tables), sizes and contents
     char *tmp = nullptr, *tab = nullptr;
-    const size_t b_src = sizeof(StripSrc) * nm, b_ofs = 4 * ((size_t)ng + 1);
-    cudaError_t e = cudaMallocAsync(&tmp, 8 + b_src + 4 * nm + 8 * (size_t)ng + b_ofs, s);
+    const size_t b_src = sizeof(StripSrc) * all, b_ofs[2] = {4 * ((size_t)ng[0] + 1), 4 * ((size_t)ng[1] + 1)};
+    const size_t b_back = 16 + 4 * all, at_ofs = (b_src + b_back + 15) / 16 * 16;
+    cudaError_t e = cudaMallocAsync(&tmp, at_ofs + b_ofs[0] + b_ofs[1] + 8 * (size_t)(ng[0] + ng[1]), s);
     if (e != cudaSuccess) { cudaGetLastError(); return; }
-    StripBuild B{};
-    B.total = reinterpret_cast<int64_t *>(tmp);
-    B.src = reinterpret_cast<StripSrc *>(tmp + 8);
-    B.far = reinterpret_cast<int32_t *>(tmp + 8 + b_src);
-    B.units = B.far + nm;
-    B.bits = reinterpret_cast<uint32_t *>(B.units + ng);
-    B.ofs = B.bits + ng;
-    B.nsrc = (int32_t)nm;
-    B.ng = ng;
-    B.trans = dir != 0;
-    B.f64 = p->dtype == SPTRSV_F64;
-    B.ring_most = strip_ring_most(B.f64, p->batched);
-    std::vector<int32_t> far(nm);
-    int64_t total = 0;
-    e = cudaMemcpyAsync(tmp + 8, src.data(), b_src, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(B.far, 0, 4 * nm, s);
-    if (e == cudaSuccess) e = strip_sizes(B, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&total, B.total, sizeof(total), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(far.data(), B.far, 4 * nm, cudaMemcpyDeviceToHost, s);
+    StripBuild B[2]{};
+    uint32_t *u = reinterpret_cast<uint32_t *>(tmp + at_ofs + b_ofs[0] + b_ofs[1]);
+    for (int d = 0; d < 2; ++d) {
+        B[d].total = reinterpret_cast<int64_t *>(tmp + b_src) + d;
+        B[d].src = reinterpret_cast<StripSrc *>(tmp) + d * nm[0];
+        B[d].far = reinterpret_cast<int32_t *>(tmp + b_src + 16) + d * nm[0];
+        B[d].ofs = reinterpret_cast<uint32_t *>(tmp + at_ofs + (d ? b_ofs[0] : 0));
+        B[d].units = reinterpret_cast<int32_t *>(u);
+        B[d].bits = u + ng[d];
+        u += 2 * ng[d];
+        B[d].nsrc = (int32_t)nm[d];
+        B[d].ng = ng[d];
+        B[d].trans = d != 0;
+        B[d].f64 = p->dtype == SPTRSV_F64;
+        B[d].ring_most = strip_ring_most(B[d].f64, p->batched);
+    }
+    std::vector<char> back(b_back);
+    int64_t total[2];
+    e = cudaMemcpyAsync(tmp, src.data(), b_src, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(tmp + b_src, 0, b_back, s);
+    for (int d = 0; d < 2 && e == cudaSuccess; ++d)
+        if (nm[d]) e = strip_sizes(B[d], s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(back.data(), tmp + b_src, b_back, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess && total > INT32_MAX) e = cudaErrorMemoryAllocation;  // (32 GB)
-    const size_t b_blocks = 16 * (size_t)total;
-    if (e == cudaSuccess) e = p->alloc_tables(&tab, b_blocks + b_ofs + 2 * (size_t)nnz);
-    if (e == cudaSuccess) {
-        uint32_t *ofs = reinterpret_cast<uint32_t *>(tab + b_blocks);
-        uint16_t *ecode = reinterpret_cast<uint16_t *>(tab + b_blocks + b_ofs);
-        e = cudaMemcpyAsync(ofs, B.ofs, b_ofs, cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess) e = strip_tables(B, ofs, reinterpret_cast<unsigned char *>(tab), ecode, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) p->release(tab);
-        for (size_t m = 0; m < nm && e == cudaSuccess; ++m)
-            mats[m]->strips[dir] = Strips{reinterpret_cast<unsigned char *>(tab), ofs + src[m].g0, ecode + src[m].e0,
-                                          strip_ring(far[m], B.ring_most)};
+    std::memcpy(total, back.data(), sizeof(total));
+    if (e == cudaSuccess && (total[0] > INT32_MAX || total[1] > INT32_MAX)) e = cudaErrorMemoryAllocation;  // (32 GB)
+    // one allocation: blocks, offsets and entry codes of both
+    const size_t b_blocks = 16 * (size_t)(total[0] + total[1]);
+    if (e == cudaSuccess)
+        e = p->alloc_tables(&tab, b_blocks + b_ofs[0] + b_ofs[1] + 2 * (size_t)(nnz[0] + nnz[1]));
+    if (e == cudaSuccess) e = cudaMemcpyAsync(tab + b_blocks, tmp + at_ofs, b_ofs[0] + b_ofs[1], cudaMemcpyDeviceToDevice, s);
+    for (int d = 0; d < 2 && e == cudaSuccess; ++d) {
+        if (!nm[d]) continue;
+        unsigned char *blocks = reinterpret_cast<unsigned char *>(tab) + (d ? 16 * (size_t)total[0] : 0);
+        uint32_t *ofs = reinterpret_cast<uint32_t *>(tab + b_blocks + (d ? b_ofs[0] : 0));
+        uint16_t *ecode = reinterpret_cast<uint16_t *>(tab + b_blocks + b_ofs[0] + b_ofs[1]) + (d ? nnz[0] : 0);
+        const int32_t *far = reinterpret_cast<const int32_t *>(back.data() + 16) + d * nm[0];
+        e = strip_tables(B[d], ofs, blocks, ecode, s);
+        for (size_t m = 0; m < nm[d] && e == cudaSuccess; ++m)
+            mats[d][m]->strips[d] = Strips{blocks, ofs + src[d * nm[0] + m].g0, ecode + src[d * nm[0] + m].e0,
+                                           strip_ring(far[m], B[d].ring_most)};
+    }
+    if (e != cudaSuccess && tab) {
+        for (int d = 0; d < 2; ++d)
+            for (PlanMat *M : mats[d]) M->strips[d] = Strips{};
+        p->release(tab);
     }
     cudaFreeAsync(tmp, s);
     if (e != cudaSuccess) cudaGetLastError();
 }
 
-// Tables of the cluster flow schedule (flow.cuh) of one direction.  One block
+// Tables of the cluster flow schedule (flow.cuh).  One block
 // of the cluster per 24 rows of the mean level: below that another block does
 // not shorten a level (power-law DAG, 63 rows a level: 2 blocks 10.4 ms, 4
 // 9.6 ms, 16 9.2 ms transpose).  Beyond 8 blocks only for very wide levels:
 // with 16 the 2D Laplacian (512 rows a level) gains 6 % at one right-hand
 // side, but the GPU holds too few such clusters for eight (5.0 against 3.5 ms).
-sptrsv_status build_flow(sptrsv_plan p, int dir)
+// The directions [d0, d1) in one go and into one allocation (as the strips).
+// The caller synchronises.
+sptrsv_status build_flow(sptrsv_plan p, int d0, int d1)
 {
     const PlanMat &M = p->M;
     const int32_t n = M.L.n, L = M.nlevels;
-    const size_t nn = (size_t)n, nc = (size_t)L * kFlowClasses;
+    const size_t nn = (size_t)n, nc = (size_t)L * kFlowClasses, nd = (size_t)(d1 - d0);
     cudaStream_t s = p->h->stream;
     const bool f64 = p->dtype == SPTRSV_F64;
     if (n > kFlowMaxRows) return SPTRSV_ENOTSUP;
@@ -585,81 +650,103 @@ sptrsv_status build_flow(sptrsv_plan p, int dir)
     while (csize < (width >= 768.0 ? kFlowMaxCluster : 8) && width > 24.0 * csize) csize <<= 1;
     while (csize > 1 && !flow_cluster_fits(csize, f64)) csize >>= 1;
     if (!flow_cluster_fits(csize, f64)) return SPTRSV_ENOTSUP;
-    const int32_t *ptr = dir ? M.d_cp : M.L.row_ptr, *idx = dir ? M.d_crow : M.L.col_idx;
-    int32_t *order = nullptr;
-    cudaError_t e = cudaMallocAsync(&order, sizeof(int32_t) * (4 * nn + nc), s);
+    // scratch: counts of all directions (read back), then by direction order,
+    // its inverse, and the positions' blocks and masks
+    int32_t *counts = nullptr;
+    cudaError_t e = cudaMallocAsync(&counts, sizeof(int32_t) * nd * (4 * nn + nc), s);
     if (e != cudaSuccess) return from_cuda(e);
-    int32_t *iperm = order + nn, *counts = iperm + 3 * nn;
-    uint32_t *meta = reinterpret_cast<uint32_t *>(iperm + nn), *mask = meta + nn;
-    e = flow_order(ptr, M.d_lev, n, L, dir != 0, order, iperm, counts, s);
-    std::vector<int32_t> cnt(nc);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(cnt.data(), counts, sizeof(int32_t) * nc, cudaMemcpyDeviceToHost, s);
+    struct Dir {
+        const int32_t *ptr, *idx;
+        int32_t *order, *iperm;
+        uint32_t *meta, *mask;
+        int32_t g0, ng;  // its groups in the list of all
+    } D[2];
+    for (int d = d0; d < d1 && e == cudaSuccess; ++d) {
+        Dir &Q = D[d - d0];
+        Q.ptr = d ? M.d_cp : M.L.row_ptr;
+        Q.idx = d ? M.d_crow : M.L.col_idx;
+        Q.order = counts + nd * nc + (size_t)(d - d0) * 4 * nn;
+        Q.iperm = Q.order + nn;
+        Q.meta = reinterpret_cast<uint32_t *>(Q.iperm + nn);
+        Q.mask = Q.meta + nn;
+        e = flow_order(Q.ptr, M.d_lev, n, L, d != 0, Q.order, Q.iperm, counts + (size_t)(d - d0) * nc, s);
+    }
+    std::vector<int32_t> cnt(nd * nc);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(cnt.data(), counts, sizeof(int32_t) * nd * nc, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     // groups of one level and class, an equal share of every level's groups,
     // in order, to each block of the cluster
-    std::vector<std::vector<FlowGroup>> by((size_t)csize);
-    std::vector<FlowGroup> lev;
-    int32_t q = 0;
-    static const int llpr[kFlowClasses] = {0, 2, 4, 5};
-    for (int32_t l = 0; l < L && e == cudaSuccess; ++l) {
-        lev.clear();
-        for (int c = 0; c < kFlowClasses; ++c) {
-            int32_t left = cnt[(size_t)l * kFlowClasses + c];
-            for (const int32_t most = 32 >> llpr[c]; left > 0;) {
-                const int32_t take = std::min(most, left);
-                lev.push_back(FlowGroup{q, take, llpr[c]});
-                q += take;
-                left -= take;
-            }
-        }
-        const int64_t G = (int64_t)lev.size();
-        for (int64_t g = 0; g < G; ++g) by[(size_t)(g * csize / G)].push_back(lev[(size_t)g]);
-    }
     std::vector<FlowGroup> all;
-    std::vector<int32_t> gptr(1, 0);
-    for (const auto &v : by) {
-        all.insert(all.end(), v.begin(), v.end());
-        gptr.push_back((int32_t)all.size());
+    std::vector<int32_t> gptr;  // csize + 1 of each direction
+    static const int llpr[kFlowClasses] = {0, 2, 4, 5};
+    for (size_t d = 0; d < nd && e == cudaSuccess; ++d) {
+        std::vector<std::vector<FlowGroup>> by((size_t)csize);
+        std::vector<FlowGroup> lev;
+        int32_t q = 0;
+        for (int32_t l = 0; l < L; ++l) {
+            lev.clear();
+            for (int c = 0; c < kFlowClasses; ++c) {
+                int32_t left = cnt[d * nc + (size_t)l * kFlowClasses + c];
+                for (const int32_t most = 32 >> llpr[c]; left > 0;) {
+                    const int32_t take = std::min(most, left);
+                    lev.push_back(FlowGroup{q, take, llpr[c]});
+                    q += take;
+                    left -= take;
+                }
+            }
+            const int64_t G = (int64_t)lev.size();
+            for (int64_t g = 0; g < G; ++g) by[(size_t)(g * csize / G)].push_back(lev[(size_t)g]);
+        }
+        D[d].g0 = (int32_t)all.size();
+        gptr.push_back(0);
+        for (const auto &v : by) {
+            all.insert(all.end(), v.begin(), v.end());
+            gptr.push_back((int32_t)all.size() - D[d].g0);
+        }
+        D[d].ng = gptr.back();
     }
     // one allocation, so that nothing is left of tables that cannot be had
     const size_t ns = 32 * std::max<size_t>(all.size(), 1), w = f64 ? 8 : 4;
     const size_t at_codes = sizeof(FlowLane) * ns, at_vals = at_codes + sizeof(uint4) * ns;
     const size_t at_inv = at_vals + 4 * w * ns, at_src = at_inv + w * ns, at_ecode = at_src + sizeof(int2) * ns;
-    const size_t at_gptr = at_ecode + sizeof(uint32_t) * (size_t)M.L.nnz;
+    const size_t at_gptr = at_ecode + sizeof(uint32_t) * (size_t)M.L.nnz * nd;
     char *tab = nullptr;
     FlowGroup *groups = nullptr;
     if (e == cudaSuccess) e = p->alloc_tables(&tab, at_gptr + sizeof(int32_t) * gptr.size());
-    FlowLane *lanes = reinterpret_cast<FlowLane *>(tab);
-    uint4 *codes = reinterpret_cast<uint4 *>(tab + at_codes);
-    int2 *src = reinterpret_cast<int2 *>(tab + at_src);
-    uint32_t *ecode = reinterpret_cast<uint32_t *>(tab + at_ecode);
-    int32_t *d_gptr = reinterpret_cast<int32_t *>(tab + at_gptr);
-    FlowSched F{};
-    F.vals = tab + at_vals;
-    F.inv = tab + at_inv;
     if (e == cudaSuccess) e = cudaMallocAsync(&groups, sizeof(FlowGroup) * std::max<size_t>(all.size(), 1), s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(groups, all.data(), sizeof(FlowGroup) * all.size(), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(d_gptr, gptr.data(), sizeof(int32_t) * gptr.size(), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
-        e = flow_tables(ptr, idx, n, dir != 0, f64, order, iperm, groups, d_gptr, (int32_t)all.size(), csize, meta,
-                        mask, lanes, codes, src, ecode, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFreeAsync(order, s);
+        e = cudaMemcpyAsync(tab + at_gptr, gptr.data(), sizeof(int32_t) * gptr.size(), cudaMemcpyHostToDevice, s);
+    for (int d = d0; d < d1 && e == cudaSuccess; ++d) {
+        const Dir &Q = D[d - d0];
+        const size_t s0 = 32 * (size_t)Q.g0;
+        FlowLane *lanes = reinterpret_cast<FlowLane *>(tab) + s0;
+        uint4 *codes = reinterpret_cast<uint4 *>(tab + at_codes) + s0;
+        int2 *src = reinterpret_cast<int2 *>(tab + at_src) + s0;
+        uint32_t *ecode = reinterpret_cast<uint32_t *>(tab + at_ecode) + (size_t)(d - d0) * (size_t)M.L.nnz;
+        const int32_t *d_gptr = reinterpret_cast<int32_t *>(tab + at_gptr) + (size_t)(d - d0) * ((size_t)csize + 1);
+        e = flow_tables(Q.ptr, Q.idx, n, d != 0, f64, Q.order, Q.iperm, groups + Q.g0, d_gptr, Q.ng, csize, Q.meta,
+                        Q.mask, lanes, codes, src, ecode, s);
+        FlowSched F{};
+        F.lanes = lanes;
+        F.codes = codes;
+        F.src = src;
+        F.ecode = ecode;
+        F.gptr = d_gptr;
+        F.vals = tab + at_vals + 4 * w * s0;
+        F.inv = tab + at_inv + w * s0;
+        F.n = n;
+        F.csize = csize;
+        F.ngroups = Q.ng;
+        p->flow[d] = F;
+    }
+    cudaFreeAsync(counts, s);
     if (groups) cudaFreeAsync(groups, s);
     if (e != cudaSuccess) {
         if (tab) p->release(tab);
         return from_cuda(e);
     }
-    F.lanes = lanes;
-    F.codes = codes;
-    F.src = src;
-    F.ecode = ecode;
-    F.gptr = d_gptr;
-    F.n = n;
-    F.csize = csize;
-    F.ngroups = (int32_t)all.size();
-    p->flow[dir] = F;
-    p->flow_ready[dir] = true;
+    for (int d = d0; d < d1; ++d) p->flow_ready[d] = true;
     return SPTRSV_OK;
 }
 
@@ -676,15 +763,24 @@ bool flow_wanted(const sptrsv_plan_st *p)
 // cannot be had, the grid-wide hybrid kernel runs.
 sptrsv_status prepare_schedules(sptrsv_plan p)
 {
-    bool grid_wide = false;
-    for (int dir = 0; dir < (p->have_csc ? 2 : 1); ++dir) {
-        if (flow_wanted(p) && !p->flow_ready[dir] && !p->flow_off[dir])
-            p->flow_off[dir] = build_flow(p, dir) != SPTRSV_OK;
-        grid_wide = grid_wide || !flow_wanted(p) || !p->flow_ready[dir];
-        if (p->mode == SPTRSV_MODE_BLOCK && p->rpw == 32 && p->M.L.n > 0 && !p->M.strips[dir].blocks)
-            build_strips(p, {&p->M}, dir);
-    }
-    return p->mode == SPTRSV_MODE_HYBRID && grid_wide ? ensure_hybrid(p) : SPTRSV_OK;
+    const int dirs = p->have_csc ? 2 : 1;
+    auto open = [&](int d) { return flow_wanted(p) && d < dirs && !p->flow_ready[d] && !p->flow_off[d]; };
+    bool built = open(0) || open(1);
+    // (where there is no room for both directions, for one)
+    if (!(open(0) && open(1)) || build_flow(p, 0, 2) != SPTRSV_OK)
+        for (int d = 0; d < dirs; ++d)
+            if (open(d)) p->flow_off[d] = build_flow(p, d, d + 1) != SPTRSV_OK;
+    std::vector<PlanMat *> need[2];
+    for (int d = 0; d < dirs; ++d)
+        if (p->mode == SPTRSV_MODE_BLOCK && p->rpw == 32 && p->M.L.n > 0 && !p->M.strips[d].blocks)
+            need[d].push_back(&p->M);
+    build_strips(p, need);
+    built = built || !need[0].empty() || !need[1].empty();
+    sptrsv_status st = SPTRSV_OK;
+    if (p->mode == SPTRSV_MODE_HYBRID && !(flow_wanted(p) && p->flow_ready[0] && p->flow_ready[dirs - 1]))
+        st = ensure_hybrid(p);
+    const cudaError_t e = built ? cudaStreamSynchronize(p->h->stream) : cudaSuccess;
+    return st == SPTRSV_OK ? from_cuda(e) : st;
 }
 
 // Mode from the mean level width: narrow (deep) systems stay on one SM, very
@@ -938,26 +1034,32 @@ extern "C" sptrsv_status sptrsv_plan_create(sptrsv_handle h, const sptrsv_csr *L
     sptrsv_plan_opts o{};
     if (opts) o = *opts;
     if (o.wait_limit_us > 0) p->spin = o.wait_limit_us * 1000;
+    const size_t nn = (size_t)(L->n > 0 ? L->n : 1);
+    p->reserve(p->padded(sizeof(PlanCtl)) + 3 * p->padded(4 * nn) + p->padded(16 * nn) + mat_bytes(*L, T, o.build_transpose != 0));
     cudaError_t e = p->alloc(&p->d_ctl, sizeof(PlanCtl));
     if (e == cudaSuccess) e = cudaMemset(p->d_ctl, 0, sizeof(PlanCtl));
-    if (e == cudaSuccess) e = p->alloc(&p->d_flags, sizeof(uint32_t) * (size_t)(L->n > 0 ? L->n : 1));
-    if (e == cudaSuccess) e = cudaMemset(p->d_flags, 0, sizeof(uint32_t) * (size_t)(L->n > 0 ? L->n : 1));
-    if (e == cudaSuccess) e = p->alloc(&p->d_vflags, 16 * (size_t)(L->n > 0 ? L->n : 1));
-    if (e == cudaSuccess) e = cudaMemset(p->d_vflags, 0, 16 * (size_t)(L->n > 0 ? L->n : 1));
+    if (e == cudaSuccess) e = p->alloc(&p->d_flags, sizeof(uint32_t) * nn);
+    if (e == cudaSuccess) e = cudaMemset(p->d_flags, 0, sizeof(uint32_t) * nn);
+    if (e == cudaSuccess) e = p->alloc(&p->d_vflags, 16 * nn);
     if (e != cudaSuccess) { sptrsv_plan_destroy(p); return from_cuda(e); }
-    st = prepare_mat(p, p->M, *L, T, o.build_transpose != 0);
+    unsigned long long nlong = 0;
+    if (!valid_rpw(o.rows_per_warp)) {
+        // (read back by the analysis' synchronisation)
+        unsigned long long *d = reinterpret_cast<unsigned long long *>(h->d_scratch + 8);
+        e = launch_count_long(L->row_ptr, L->n, 32, d, h->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&nlong, d, sizeof(nlong), cudaMemcpyDeviceToHost, h->stream);
+        if (e == cudaSuccess && L->n == 0) e = cudaStreamSynchronize(h->stream);
+        if (e != cudaSuccess) { sptrsv_plan_destroy(p); return from_cuda(e); }
+    }
+    // (the level costs go where the flags will be)
+    st = prepare_mat(p, p->M, *L, T, o.build_transpose != 0, reinterpret_cast<int64_t *>(p->d_vflags));
+    if (st == SPTRSV_OK) st = from_cuda(cudaMemsetAsync(p->d_vflags, 0, 16 * nn, h->stream));
     if (st != SPTRSV_OK) { sptrsv_plan_destroy(p); return st; }
     p->have_csc = o.build_transpose != 0;
     p->mode = o.mode != SPTRSV_MODE_AUTO ? o.mode : auto_mode(p->M);
     if (valid_rpw(o.rows_per_warp)) {
         p->rpw = o.rows_per_warp;
     } else {
-        unsigned long long nlong = 0;
-        unsigned long long *d = reinterpret_cast<unsigned long long *>(h->d_scratch + 8);
-        cudaError_t e = launch_count_long(L->row_ptr, L->n, 32, d, h->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&nlong, d, sizeof(nlong), cudaMemcpyDeviceToHost, h->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-        if (e != cudaSuccess) { sptrsv_plan_destroy(p); return from_cuda(e); }
         p->rpw = p->mode == SPTRSV_MODE_BLOCK ? block_rpw(L->n, L->nnz, (int64_t)nlong)
                                               : default_rpw(L->n, L->nnz, (int64_t)nlong);
     }
@@ -980,9 +1082,10 @@ extern "C" sptrsv_status sptrsv_plan_create(sptrsv_handle h, const sptrsv_csr *L
     }
     p->grid_sf = persistent_grid_syncfree(1, p->dtype == SPTRSV_F64, h->di);
     st = ensure_chunks(p);
+    // (what the solves cannot do without they ask for again)
+    if (st == SPTRSV_OK) prepare_schedules(p);
     if (st == SPTRSV_OK) st = from_cuda(cudaStreamSynchronize(h->stream));
     if (st != SPTRSV_OK) { sptrsv_plan_destroy(p); return st; }
-    prepare_schedules(p);  // (what the solves cannot do without they ask for again)
     *plan = p;
     return SPTRSV_OK;
 }
@@ -1194,12 +1297,10 @@ sptrsv_status rebuild_items(sptrsv_plan p, int dir)
     std::vector<double> est;
     size_t smem = 16;
     G.csc_vals = G.strips = false;
-    auto takes_strips = [&](int m) { return G.rpw[m] == 32 && G.sched[m] == kSchedInOrder && p->mats[m].L.n > 0; };
-    std::vector<PlanMat *> need;
-    if (dir == 0 || p->have_csc)
-        for (int m = 0; m < nmat; ++m)
-            if (takes_strips(m) && !p->mats[m].strips[dir].blocks) need.push_back(&p->mats[m]);
-    if (!need.empty()) build_strips(p, need, dir);
+    auto takes_strips = [&](int m) { return p->takes_strips(dir, m); };
+    std::vector<PlanMat *> need[2];
+    p->strips_to_build(dir, &need[dir]);
+    build_strips(p, need);
     // (only systems solved over them: the others' values need not be laid out
     // before every solve)
     bool changed = false;
@@ -1392,8 +1493,19 @@ extern "C" sptrsv_status sptrsv_batch_plan_create(sptrsv_handle h, int32_t nmat,
     bool want_csc = false;
     for (int m = 0; m < nmat && opts; ++m) want_csc = want_csc || opts[m].build_transpose;
     if (opts && opts[0].wait_limit_us > 0) p->spin = opts[0].wait_limit_us * 1000;
+    size_t mats_bytes = 0;
+    int32_t n_most = 1;
+    for (int m = 0; m < nmat; ++m) {
+        if (check_csr(&Ls[m]) != SPTRSV_OK) continue;  // (refused below)
+        mats_bytes += mat_bytes(Ls[m], Ts ? &Ts[m] : nullptr, want_csc);
+        n_most = std::max(n_most, Ls[m].n);
+    }
+    p->reserve(p->padded(sizeof(PlanCtl)) + mats_bytes);
     cudaError_t e = p->alloc(&p->d_ctl, sizeof(PlanCtl));
     if (e == cudaSuccess) e = cudaMemset(p->d_ctl, 0, sizeof(PlanCtl));
+    if (e != cudaSuccess) { sptrsv_plan_destroy(p); return from_cuda(e); }
+    DeviceArray<int64_t> cost;
+    e = cost.get((size_t)n_most);
     if (e != cudaSuccess) { sptrsv_plan_destroy(p); return from_cuda(e); }
     p->mats.resize((size_t)nmat);
     p->rhs_off.assign((size_t)nmat + 1, 0);
@@ -1416,7 +1528,7 @@ extern "C" sptrsv_status sptrsv_batch_plan_create(sptrsv_handle h, int32_t nmat,
             st = SPTRSV_EINVAL;
         if (st == SPTRSV_OK && opts && opts[m].rhs_tile != 0 && !valid_tile(opts[m].rhs_tile))
             st = SPTRSV_EINVAL;
-        if (st == SPTRSV_OK) st = prepare_mat(p, p->mats[m], Ls[m], Ts ? &Ts[m] : nullptr, want_csc);
+        if (st == SPTRSV_OK) st = prepare_mat(p, p->mats[m], Ls[m], Ts ? &Ts[m] : nullptr, want_csc, cost.p);
         if (st != SPTRSV_OK) { sptrsv_plan_destroy(p); return st; }
         const PlanMat &M = p->mats[m];
         BatchMat &B = p->h_mats[m];
@@ -1499,6 +1611,9 @@ extern "C" sptrsv_status sptrsv_batch_plan_create(sptrsv_handle h, int32_t nmat,
             e = cudaMemcpy(p->d_tchunks, t.data(), sizeof(RowChunk) * t.size(), cudaMemcpyHostToDevice);
         if (e != cudaSuccess) { sptrsv_plan_destroy(p); return from_cuda(e); }
     }
+    std::vector<PlanMat *> need[2];
+    for (int d = 0; d < 2; ++d) p->strips_to_build(d, &need[d]);
+    build_strips(p, need);
     sptrsv_status st = rebuild_items(p, 0);
     if (st == SPTRSV_OK) st = rebuild_items(p, 1);
     if (st != SPTRSV_OK) { sptrsv_plan_destroy(p); return st; }
