@@ -687,27 +687,26 @@ cudaError_t launch_level_stats(int32_t n, int64_t nnz, int32_t nlevels, const in
 }
 
 cudaError_t level_partition(const sptrsv_csr &L, const int32_t *lev, int32_t nlevels,
-                            int32_t *perm, int32_t *level_ptr, int64_t *cost, cudaStream_t s)
+                            int32_t *perm, int32_t *level_ptr, int64_t *cost, cudaStream_t s,
+                            const Scratch *from)
 {
     const int32_t n = L.n;
     if (n <= 0) return cudaMemsetAsync(level_ptr, 0, sizeof(int32_t), s);
     int32_t *counts = nullptr, *iota = nullptr;
     uint32_t *keys_out = nullptr;
-    cudaError_t e = cudaMallocAsync(&counts, sizeof(int32_t) * (size_t)nlevels, s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&iota, sizeof(int32_t) * (size_t)n, s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&keys_out, sizeof(uint32_t) * (size_t)n, s);
+    Scratch tmp(s, from);
+    cudaError_t e = tmp.take(&counts, (size_t)nlevels);
+    if (e == cudaSuccess) e = tmp.take(&iota, (size_t)n);
+    if (e == cudaSuccess) e = tmp.take(&keys_out, (size_t)n);
     if (e != cudaSuccess) return e;
     e = launch_level_hist(L, lev, nlevels, counts, cost, s);
-    if (e == cudaSuccess) e = exclusive_scan_i32(counts, level_ptr, nlevels, nullptr, s);
+    if (e == cudaSuccess) e = exclusive_scan_i32(counts, level_ptr, nlevels, nullptr, s, &tmp);
     if (e == cudaSuccess) {
         k_iota<<<grid_for(n, 256), 256, 0, s>>>(iota, n);
         int bits = 0;
         while (bits < 32 && ((uint32_t)(nlevels - 1) >> bits) != 0) ++bits;
-        e = radix_sort_pairs((const uint32_t *)lev, iota, keys_out, perm, n, bits, s);
+        e = radix_sort_pairs((const uint32_t *)lev, iota, keys_out, perm, n, bits, s, &tmp);
     }
-    cudaFreeAsync(counts, s);
-    cudaFreeAsync(iota, s);
-    cudaFreeAsync(keys_out, s);
     return e;
 }
 

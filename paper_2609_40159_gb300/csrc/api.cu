@@ -401,12 +401,12 @@ sptrsv_status levels_impl(sptrsv_handle h, const sptrsv_csr &L, int32_t *lev, in
 
 sptrsv_status analyze_into(sptrsv_handle h, const sptrsv_csr &L, int32_t *lev, int32_t *perm,
                            int32_t *level_ptr, int64_t *cost, int32_t *nlevels, double *stats,
-                           long long spin, int32_t first_row = 0)
+                           long long spin, int32_t first_row = 0, const Scratch *from = nullptr)
 {
     sptrsv_status st = levels_impl(h, L, lev, nlevels, spin, first_row);
     if (st != SPTRSV_OK) return st;
     cudaStream_t s = h->stream;
-    cudaError_t e = level_partition(L, lev, *nlevels, perm, level_ptr, cost, s);
+    cudaError_t e = level_partition(L, lev, *nlevels, perm, level_ptr, cost, s, from);
     if (e == cudaSuccess && stats) {
         double *dst = reinterpret_cast<double *>(h->d_scratch + 2);
         e = launch_level_stats(L.n, L.nnz, *nlevels, level_ptr, cost, dst, s);
@@ -443,10 +443,21 @@ size_t mat_bytes(const sptrsv_csr &L, const sptrsv_csr *T, bool want_csc)
     return all;
 }
 
+// Scratch of a plan's steps (a system of n rows and nnz entries): the sort by
+// level, the sort by column, and both directions' orders of the cluster flow.
+size_t plan_scratch(int32_t n, int64_t nnz, bool want_csc)
+{
+    auto b = [](int64_t count) { return Scratch::padded(4 * (size_t)std::max<int64_t>(count, 1)); };
+    const size_t rows = 3 * b(n) + b(3 * (int64_t)n) + radix_sort_scratch(n);
+    const size_t csc = want_csc ? b(n) + 3 * b(nnz) + radix_sort_scratch(nnz) : 0;
+    const size_t flow = b((want_csc ? 2 : 1) * (int64_t)n * 5) + b(3 * (int64_t)n) + radix_sort_scratch(n);
+    return std::max({rows, csc, flow});
+}
+
 // Analysis + schedule data + optional CSC for one system of a plan; cost:
 // scratch for the level costs (n entries).  The caller synchronises.
 sptrsv_status prepare_mat(sptrsv_plan p, PlanMat &M, const sptrsv_csr &L, const sptrsv_csr *T,
-                          bool want_csc, int64_t *cost)
+                          bool want_csc, int64_t *cost, const Scratch *from)
 {
     sptrsv_handle h = p->h;
     cudaStream_t s = h->stream;
@@ -463,7 +474,7 @@ sptrsv_status prepare_mat(sptrsv_plan p, PlanMat &M, const sptrsv_csr &L, const 
     if (e == cudaSuccess) e = p->alloc(&M.d_perm, sizeof(int32_t) * nn);
     if (e == cudaSuccess) e = p->alloc(&M.d_level_ptr, sizeof(int32_t) * (nn + 1));
     if (e != cudaSuccess) return from_cuda(e);
-    sptrsv_status st = analyze_into(h, L, M.d_lev, M.d_perm, M.d_level_ptr, cost, &M.nlevels, nullptr, p->spin);
+    sptrsv_status st = analyze_into(h, L, M.d_lev, M.d_perm, M.d_level_ptr, cost, &M.nlevels, nullptr, p->spin, 0, from);
     if (st != SPTRSV_OK) return st;
     M.h_level_ptr.assign((size_t)M.nlevels + 1, 0);
     if (n > 0) {
@@ -479,7 +490,7 @@ sptrsv_status prepare_mat(sptrsv_plan p, PlanMat &M, const sptrsv_csr &L, const 
         if (e == cudaSuccess) e = p->alloc(&M.d_ttmap, sizeof(int32_t) * tnz);
         if (e == cudaSuccess) e = p->alloc(&M.d_tcmask, sizeof(uint32_t) * ((nn + 31) / 32));
         if (e == cudaSuccess)
-            e = M.T.nnz > 0 ? build_csc(M.T.row_ptr, M.T.col_idx, n, M.T.nnz, M.d_tcp, M.d_trow, M.d_ttmap, s)
+            e = M.T.nnz > 0 ? build_csc(M.T.row_ptr, M.T.col_idx, n, M.T.nnz, M.d_tcp, M.d_trow, M.d_ttmap, s, from)
                             : cudaMemsetAsync(M.d_tcp, 0, sizeof(int32_t) * (nn + 1), s);
         if (e == cudaSuccess) e = build_tmask(M.d_tcp, n, M.d_tcmask, s);
         if (e != cudaSuccess) return from_cuda(e);
@@ -490,7 +501,7 @@ sptrsv_status prepare_mat(sptrsv_plan p, PlanMat &M, const sptrsv_csr &L, const 
         if (e == cudaSuccess) e = p->alloc(&M.d_tmap, sizeof(int32_t) * (size_t)(L.nnz > 0 ? L.nnz : 1));
         if (e == cudaSuccess)
             e = p->alloc(&M.d_cv, (L.dtype == SPTRSV_F64 ? 8 : 4) * (size_t)(L.nnz > 0 ? L.nnz : 1));
-        if (e == cudaSuccess) e = build_csc(L.row_ptr, L.col_idx, n, L.nnz, M.d_cp, M.d_crow, M.d_tmap, s);
+        if (e == cudaSuccess) e = build_csc(L.row_ptr, L.col_idx, n, L.nnz, M.d_cp, M.d_crow, M.d_tmap, s, from);
         if (e != cudaSuccess) return from_cuda(e);
     }
     return SPTRSV_OK;
@@ -554,10 +565,9 @@ sptrsv_status ensure_hybrid(sptrsv_plan p)
 
 // Strips (strip.cuh) of the systems of each direction that have none; left out
 // when their memory cannot be had (then the solves take several lanes per row).
-// Both directions in one go, as of a small system the allocations (40 us for
-// one from the stream's pool, and as much again when a synchronisation gives
-// it back) and synchronisations are what this takes.  The caller synchronises.
-void build_strips(sptrsv_plan p, const std::vector<PlanMat *> (&mats)[2])
+// Both directions in one go, as of a small system the allocations and
+// synchronisations are what this takes.  The caller synchronises.
+void build_strips(sptrsv_plan p, const std::vector<PlanMat *> (&mats)[2], const Scratch *from = nullptr)
 {
     const size_t nm[2] = {mats[0].size(), mats[1].size()}, all = nm[0] + nm[1];
     if (all == 0) return;
@@ -576,7 +586,8 @@ void build_strips(sptrsv_plan p, const std::vector<PlanMat *> (&mats)[2])
     char *tmp = nullptr, *tab = nullptr;
     const size_t b_src = sizeof(StripSrc) * all, b_ofs[2] = {4 * ((size_t)ng[0] + 1), 4 * ((size_t)ng[1] + 1)};
     const size_t b_back = 16 + 4 * all, at_ofs = (b_src + b_back + 15) / 16 * 16;
-    cudaError_t e = cudaMallocAsync(&tmp, at_ofs + b_ofs[0] + b_ofs[1] + 8 * (size_t)(ng[0] + ng[1]), s);
+    Scratch scratch(s, from);
+    cudaError_t e = scratch.take(&tmp, at_ofs + b_ofs[0] + b_ofs[1] + 8 * (size_t)(ng[0] + ng[1]));
     if (e != cudaSuccess) { cudaGetLastError(); return; }
     StripBuild B[2]{};
     uint32_t *u = reinterpret_cast<uint32_t *>(tmp + at_ofs + b_ofs[0] + b_ofs[1]);
@@ -599,7 +610,7 @@ void build_strips(sptrsv_plan p, const std::vector<PlanMat *> (&mats)[2])
     e = cudaMemcpyAsync(tmp, src.data(), b_src, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(tmp + b_src, 0, b_back, s);
     for (int d = 0; d < 2 && e == cudaSuccess; ++d)
-        if (nm[d]) e = strip_sizes(B[d], s);
+        if (nm[d]) e = strip_sizes(B[d], s, &scratch);
     if (e == cudaSuccess) e = cudaMemcpyAsync(back.data(), tmp + b_src, b_back, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     std::memcpy(total, back.data(), sizeof(total));
@@ -625,7 +636,6 @@ void build_strips(sptrsv_plan p, const std::vector<PlanMat *> (&mats)[2])
             for (PlanMat *M : mats[d]) M->strips[d] = Strips{};
         p->release(tab);
     }
-    cudaFreeAsync(tmp, s);
     if (e != cudaSuccess) cudaGetLastError();
 }
 
@@ -637,7 +647,7 @@ void build_strips(sptrsv_plan p, const std::vector<PlanMat *> (&mats)[2])
 // side, but the GPU holds too few such clusters for eight (5.0 against 3.5 ms).
 // The directions [d0, d1) in one go and into one allocation (as the strips).
 // The caller synchronises.
-sptrsv_status build_flow(sptrsv_plan p, int d0, int d1)
+sptrsv_status build_flow(sptrsv_plan p, int d0, int d1, const Scratch *from)
 {
     const PlanMat &M = p->M;
     const int32_t n = M.L.n, L = M.nlevels;
@@ -653,7 +663,8 @@ sptrsv_status build_flow(sptrsv_plan p, int d0, int d1)
     // scratch: counts of all directions (read back), then by direction order,
     // its inverse, and the positions' blocks and masks
     int32_t *counts = nullptr;
-    cudaError_t e = cudaMallocAsync(&counts, sizeof(int32_t) * nd * (4 * nn + nc), s);
+    Scratch scratch(s, from);
+    cudaError_t e = scratch.take(&counts, nd * (4 * nn + nc));
     if (e != cudaSuccess) return from_cuda(e);
     struct Dir {
         const int32_t *ptr, *idx;
@@ -669,7 +680,7 @@ sptrsv_status build_flow(sptrsv_plan p, int d0, int d1)
         Q.iperm = Q.order + nn;
         Q.meta = reinterpret_cast<uint32_t *>(Q.iperm + nn);
         Q.mask = Q.meta + nn;
-        e = flow_order(Q.ptr, M.d_lev, n, L, d != 0, Q.order, Q.iperm, counts + (size_t)(d - d0) * nc, s);
+        e = flow_order(Q.ptr, M.d_lev, n, L, d != 0, Q.order, Q.iperm, counts + (size_t)(d - d0) * nc, s, &scratch);
     }
     std::vector<int32_t> cnt(nd * nc);
     if (e == cudaSuccess) e = cudaMemcpyAsync(cnt.data(), counts, sizeof(int32_t) * nd * nc, cudaMemcpyDeviceToHost, s);
@@ -713,7 +724,7 @@ sptrsv_status build_flow(sptrsv_plan p, int d0, int d1)
     char *tab = nullptr;
     FlowGroup *groups = nullptr;
     if (e == cudaSuccess) e = p->alloc_tables(&tab, at_gptr + sizeof(int32_t) * gptr.size());
-    if (e == cudaSuccess) e = cudaMallocAsync(&groups, sizeof(FlowGroup) * std::max<size_t>(all.size(), 1), s);
+    if (e == cudaSuccess) e = scratch.take(&groups, all.size());
     if (e == cudaSuccess) e = cudaMemcpyAsync(groups, all.data(), sizeof(FlowGroup) * all.size(), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(tab + at_gptr, gptr.data(), sizeof(int32_t) * gptr.size(), cudaMemcpyHostToDevice, s);
@@ -740,8 +751,6 @@ sptrsv_status build_flow(sptrsv_plan p, int d0, int d1)
         F.ngroups = Q.ng;
         p->flow[d] = F;
     }
-    cudaFreeAsync(counts, s);
-    if (groups) cudaFreeAsync(groups, s);
     if (e != cudaSuccess) {
         if (tab) p->release(tab);
         return from_cuda(e);
@@ -761,20 +770,20 @@ bool flow_wanted(const sptrsv_plan_st *p)
 // Builds the tables of the plan's mode and settings, so that a solve launches
 // kernels only: called by whatever changes them.  Where the flow's tables
 // cannot be had, the grid-wide hybrid kernel runs.
-sptrsv_status prepare_schedules(sptrsv_plan p)
+sptrsv_status prepare_schedules(sptrsv_plan p, const Scratch *from = nullptr)
 {
     const int dirs = p->have_csc ? 2 : 1;
     auto open = [&](int d) { return flow_wanted(p) && d < dirs && !p->flow_ready[d] && !p->flow_off[d]; };
     bool built = open(0) || open(1);
     // (where there is no room for both directions, for one)
-    if (!(open(0) && open(1)) || build_flow(p, 0, 2) != SPTRSV_OK)
+    if (!(open(0) && open(1)) || build_flow(p, 0, 2, from) != SPTRSV_OK)
         for (int d = 0; d < dirs; ++d)
-            if (open(d)) p->flow_off[d] = build_flow(p, d, d + 1) != SPTRSV_OK;
+            if (open(d)) p->flow_off[d] = build_flow(p, d, d + 1, from) != SPTRSV_OK;
     std::vector<PlanMat *> need[2];
     for (int d = 0; d < dirs; ++d)
         if (p->mode == SPTRSV_MODE_BLOCK && p->rpw == 32 && p->M.L.n > 0 && !p->M.strips[d].blocks)
             need[d].push_back(&p->M);
-    build_strips(p, need);
+    build_strips(p, need, from);
     built = built || !need[0].empty() || !need[1].empty();
     sptrsv_status st = SPTRSV_OK;
     if (p->mode == SPTRSV_MODE_HYBRID && !(flow_wanted(p) && p->flow_ready[0] && p->flow_ready[dirs - 1]))
@@ -1051,8 +1060,12 @@ extern "C" sptrsv_status sptrsv_plan_create(sptrsv_handle h, const sptrsv_csr *L
         if (e == cudaSuccess && L->n == 0) e = cudaStreamSynchronize(h->stream);
         if (e != cudaSuccess) { sptrsv_plan_destroy(p); return from_cuda(e); }
     }
+    DeviceArray<char> buffer;
+    const size_t bytes = plan_scratch(L->n, L->nnz, o.build_transpose != 0);
+    if (buffer.get(bytes) != cudaSuccess) cudaGetLastError();  // (then from the pool)
+    const Scratch scratch(h->stream, buffer.p, bytes);
     // (the level costs go where the flags will be)
-    st = prepare_mat(p, p->M, *L, T, o.build_transpose != 0, reinterpret_cast<int64_t *>(p->d_vflags));
+    st = prepare_mat(p, p->M, *L, T, o.build_transpose != 0, reinterpret_cast<int64_t *>(p->d_vflags), &scratch);
     if (st == SPTRSV_OK) st = from_cuda(cudaMemsetAsync(p->d_vflags, 0, 16 * nn, h->stream));
     if (st != SPTRSV_OK) { sptrsv_plan_destroy(p); return st; }
     p->have_csc = o.build_transpose != 0;
@@ -1083,7 +1096,7 @@ extern "C" sptrsv_status sptrsv_plan_create(sptrsv_handle h, const sptrsv_csr *L
     p->grid_sf = persistent_grid_syncfree(1, p->dtype == SPTRSV_F64, h->di);
     st = ensure_chunks(p);
     // (what the solves cannot do without they ask for again)
-    if (st == SPTRSV_OK) prepare_schedules(p);
+    if (st == SPTRSV_OK) prepare_schedules(p, &scratch);
     if (st == SPTRSV_OK) st = from_cuda(cudaStreamSynchronize(h->stream));
     if (st != SPTRSV_OK) { sptrsv_plan_destroy(p); return st; }
     *plan = p;
@@ -1493,19 +1506,25 @@ extern "C" sptrsv_status sptrsv_batch_plan_create(sptrsv_handle h, int32_t nmat,
     bool want_csc = false;
     for (int m = 0; m < nmat && opts; ++m) want_csc = want_csc || opts[m].build_transpose;
     if (opts && opts[0].wait_limit_us > 0) p->spin = opts[0].wait_limit_us * 1000;
-    size_t mats_bytes = 0;
+    size_t mats_bytes = 0, bytes = 0;
     int32_t n_most = 1;
     for (int m = 0; m < nmat; ++m) {
         if (check_csr(&Ls[m]) != SPTRSV_OK) continue;  // (refused below)
         mats_bytes += mat_bytes(Ls[m], Ts ? &Ts[m] : nullptr, want_csc);
         n_most = std::max(n_most, Ls[m].n);
+        bytes = std::max(bytes, plan_scratch(Ls[m].n, Ls[m].nnz, want_csc));
     }
     p->reserve(p->padded(sizeof(PlanCtl)) + mats_bytes);
     cudaError_t e = p->alloc(&p->d_ctl, sizeof(PlanCtl));
     if (e == cudaSuccess) e = cudaMemset(p->d_ctl, 0, sizeof(PlanCtl));
     if (e != cudaSuccess) { sptrsv_plan_destroy(p); return from_cuda(e); }
-    DeviceArray<int64_t> cost;
-    e = cost.get((size_t)n_most);
+    // scratch of every system in turn, its level costs first
+    DeviceArray<char> buffer;
+    bytes += Scratch::padded(sizeof(int64_t) * (size_t)n_most);
+    if (buffer.get(bytes) != cudaSuccess) cudaGetLastError();  // (then from the pool)
+    Scratch scratch(h->stream, buffer.p, bytes);
+    int64_t *cost = nullptr;
+    e = scratch.take(&cost, (size_t)n_most);
     if (e != cudaSuccess) { sptrsv_plan_destroy(p); return from_cuda(e); }
     p->mats.resize((size_t)nmat);
     p->rhs_off.assign((size_t)nmat + 1, 0);
@@ -1528,7 +1547,7 @@ extern "C" sptrsv_status sptrsv_batch_plan_create(sptrsv_handle h, int32_t nmat,
             st = SPTRSV_EINVAL;
         if (st == SPTRSV_OK && opts && opts[m].rhs_tile != 0 && !valid_tile(opts[m].rhs_tile))
             st = SPTRSV_EINVAL;
-        if (st == SPTRSV_OK) st = prepare_mat(p, p->mats[m], Ls[m], Ts ? &Ts[m] : nullptr, want_csc, cost.p);
+        if (st == SPTRSV_OK) st = prepare_mat(p, p->mats[m], Ls[m], Ts ? &Ts[m] : nullptr, want_csc, cost, &scratch);
         if (st != SPTRSV_OK) { sptrsv_plan_destroy(p); return st; }
         const PlanMat &M = p->mats[m];
         BatchMat &B = p->h_mats[m];
@@ -1613,7 +1632,7 @@ extern "C" sptrsv_status sptrsv_batch_plan_create(sptrsv_handle h, int32_t nmat,
     }
     std::vector<PlanMat *> need[2];
     for (int d = 0; d < 2; ++d) p->strips_to_build(d, &need[d]);
-    build_strips(p, need);
+    build_strips(p, need, &scratch);
     sptrsv_status st = rebuild_items(p, 0);
     if (st == SPTRSV_OK) st = rebuild_items(p, 1);
     if (st != SPTRSV_OK) { sptrsv_plan_destroy(p); return st; }

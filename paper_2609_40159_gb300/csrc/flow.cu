@@ -568,22 +568,22 @@ template <class T> bool flow_fits(int csize)
 bool flow_cluster_fits(int csize, bool f64) { return f64 ? flow_fits<double>(csize) : flow_fits<float>(csize); }
 
 cudaError_t flow_order(const int32_t *ptr, const int32_t *lev, int32_t n, int32_t L, bool trans, int32_t *order,
-                       int32_t *iperm, int32_t *counts, cudaStream_t s)
+                       int32_t *iperm, int32_t *counts, cudaStream_t s, const Scratch *from)
 {
     uint32_t *keys = nullptr;  // keys, sorted keys, rows
     cudaError_t e = cudaMemsetAsync(counts, 0, sizeof(int32_t) * (size_t)L * kFlowClasses, s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&keys, sizeof(uint32_t) * 3 * (size_t)n, s);
+    Scratch tmp(s, from);
+    if (e == cudaSuccess) e = tmp.take(&keys, 3 * (size_t)n);
     if (e != cudaSuccess) return e;
     int32_t *rows = reinterpret_cast<int32_t *>(keys + 2 * (size_t)n);
     k_flow_keys<<<flow_grid(n), 256, 0, s>>>(ptr, lev, n, L, trans, keys, rows, counts);
     int bits = 0;
     while (bits < 32 && (((uint32_t)L * kFlowClasses - 1) >> bits) != 0) ++bits;
-    e = radix_sort_pairs(keys, rows, keys + n, order, n, bits, s);
+    e = radix_sort_pairs(keys, rows, keys + n, order, n, bits, s, &tmp);
     if (e == cudaSuccess) {
         k_flow_inverse<<<flow_grid(n), 256, 0, s>>>(order, n, iperm);
         e = cudaGetLastError();
     }
-    cudaFreeAsync(keys, s);
     return e;
 }
 

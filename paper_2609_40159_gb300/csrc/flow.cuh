@@ -45,7 +45,7 @@ constexpr int64_t kFlowMaxRows = 900 * 1000 * 1000;  // generations of a slot fi
 // counts: L * kFlowClasses (rows per level and class); meta, mask: n entries
 // of scratch.
 cudaError_t flow_order(const int32_t *ptr, const int32_t *lev, int32_t n, int32_t L, bool trans, int32_t *order,
-                       int32_t *iperm, int32_t *counts, cudaStream_t s);
+                       int32_t *iperm, int32_t *counts, cudaStream_t s, const Scratch *from);
 cudaError_t flow_tables(const int32_t *ptr, const int32_t *idx, int32_t n, bool trans, bool f64, const int32_t *order,
                         const int32_t *iperm, const FlowGroup *groups, const int32_t *gptr, int32_t ngroups,
                         int32_t csize, uint32_t *meta, uint32_t *mask, FlowLane *lanes, uint4 *codes, int2 *src,

@@ -96,7 +96,7 @@ __global__ void k_scan_apply(const int32_t *in, int32_t *out, int64_t n, const l
 }  // namespace
 
 cudaError_t exclusive_scan_i32(const int32_t *in, int32_t *out, int64_t n, int64_t *total_dev,
-                               cudaStream_t s)
+                               cudaStream_t s, const Scratch *from)
 {
     if (n <= 0) {
         cudaError_t e = cudaMemsetAsync(out, 0, sizeof(int32_t), s);
@@ -104,15 +104,14 @@ cudaError_t exclusive_scan_i32(const int32_t *in, int32_t *out, int64_t n, int64
         return e;
     }
     const int nb = (int)((n + kScanTile - 1) / kScanTile);
+    Scratch tmp(s, from);
     long long *partial = nullptr;
-    cudaError_t e = cudaMallocAsync(&partial, sizeof(long long) * nb, s);
+    cudaError_t e = tmp.take(&partial, (size_t)nb);
     if (e != cudaSuccess) return e;
     k_scan_reduce<<<nb, kScanThreads, 0, s>>>(in, n, partial);
     k_scan_partials<<<1, kScanThreads, 0, s>>>(partial, nb, total_dev);
     k_scan_apply<<<nb, kScanThreads, 0, s>>>(in, out, n, partial);
-    e = cudaGetLastError();
-    cudaFreeAsync(partial, s);
-    return e;
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------- radix sort
@@ -182,7 +181,7 @@ __global__ void k_radix_scatter(const uint32_t *keys, const int32_t *vals, int64
 }  // namespace
 
 cudaError_t radix_sort_pairs(const uint32_t *keys, const int32_t *vals, uint32_t *keys_out,
-                             int32_t *vals_out, int64_t n, int key_bits, cudaStream_t s)
+                             int32_t *vals_out, int64_t n, int key_bits, cudaStream_t s, const Scratch *from)
 {
     if (n <= 0) return cudaSuccess;
     const int passes = key_bits <= 0 ? 1 : (key_bits + 7) / 8;
@@ -190,10 +189,11 @@ cudaError_t radix_sort_pairs(const uint32_t *keys, const int32_t *vals, uint32_t
     int32_t *hist = nullptr, *offs = nullptr;
     uint32_t *kbuf = nullptr;
     int32_t *vbuf = nullptr;
-    cudaError_t e = cudaMallocAsync(&hist, sizeof(int32_t) * 256 * (size_t)nb, s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&offs, sizeof(int32_t) * (256 * (size_t)nb + 1), s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&kbuf, sizeof(uint32_t) * (size_t)n, s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&vbuf, sizeof(int32_t) * (size_t)n, s);
+    Scratch tmp(s, from);
+    cudaError_t e = tmp.take(&hist, 256 * (size_t)nb);
+    if (e == cudaSuccess) e = tmp.take(&offs, 256 * (size_t)nb + 1);
+    if (e == cudaSuccess) e = tmp.take(&kbuf, (size_t)n);
+    if (e == cudaSuccess) e = tmp.take(&vbuf, (size_t)n);
     if (e != cudaSuccess) return e;
     // ping-pong so that the last pass writes keys_out / vals_out
     const uint32_t *ksrc = keys;
@@ -203,18 +203,21 @@ cudaError_t radix_sort_pairs(const uint32_t *keys, const int32_t *vals, uint32_t
         uint32_t *kdst = to_out ? keys_out : kbuf;
         int32_t *vdst = to_out ? vals_out : vbuf;
         k_radix_hist<<<nb, kRadixThreads, 0, s>>>(ksrc, n, 8 * p, hist, nb);
-        e = exclusive_scan_i32(hist, offs, 256 * (int64_t)nb, nullptr, s);
+        e = exclusive_scan_i32(hist, offs, 256 * (int64_t)nb, nullptr, s, &tmp);
         if (e != cudaSuccess) break;
         k_radix_scatter<<<nb, kRadixThreads, 0, s>>>(ksrc, vsrc, n, 8 * p, offs, nb, kdst, vdst);
         ksrc = kdst;
         vsrc = vdst;
     }
     if (e == cudaSuccess) e = cudaGetLastError();
-    cudaFreeAsync(hist, s);
-    cudaFreeAsync(offs, s);
-    cudaFreeAsync(kbuf, s);
-    cudaFreeAsync(vbuf, s);
     return e;
+}
+
+size_t radix_sort_scratch(int64_t n)
+{
+    const size_t nb = (size_t)((n + kRadixTile - 1) / kRadixTile), m = (size_t)std::max<int64_t>(n, 1);
+    return 2 * Scratch::padded(4 * m) + 2 * Scratch::padded(4 * (256 * nb + 1)) +
+           Scratch::padded(8 * ((256 * nb + kScanTile - 1) / kScanTile + 1));
 }
 
 // ------------------------------------------------------------ expand rows
@@ -280,34 +283,31 @@ int grid_of(int64_t work)
 // ascending inside a column, so the diagonal comes first) and the CSR
 // position of every entry tmap[nnz] -- a stable sort of the entries by column.
 cudaError_t build_csc(const int32_t *rp, const int32_t *ci, int32_t n, int64_t nnz, int32_t *cp,
-                      int32_t *crow, int32_t *tmap, cudaStream_t s)
+                      int32_t *crow, int32_t *tmap, cudaStream_t s, const Scratch *from)
 {
     if (n <= 0) return cudaMemsetAsync(cp, 0, sizeof(int32_t), s);
     int32_t *cnt = nullptr, *iota = nullptr, *erow = nullptr;
     uint32_t *kout = nullptr;
-    cudaError_t e = cudaMallocAsync(&cnt, sizeof(int32_t) * (size_t)n, s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&iota, sizeof(int32_t) * (size_t)nnz, s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&erow, sizeof(int32_t) * (size_t)nnz, s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&kout, sizeof(uint32_t) * (size_t)nnz, s);
+    Scratch tmp(s, from);
+    cudaError_t e = tmp.take(&cnt, (size_t)n);
+    if (e == cudaSuccess) e = tmp.take(&iota, (size_t)nnz);
+    if (e == cudaSuccess) e = tmp.take(&erow, (size_t)nnz);
+    if (e == cudaSuccess) e = tmp.take(&kout, (size_t)nnz);
     if (e != cudaSuccess) return e;
     cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)n, s);
     k_col_count<<<grid_of(nnz), 256, 0, s>>>(ci, nnz, cnt);
-    e = exclusive_scan_i32(cnt, cp, n, nullptr, s);
+    e = exclusive_scan_i32(cnt, cp, n, nullptr, s, &tmp);
     if (e == cudaSuccess) {
         k_iota32<<<grid_of(nnz), 256, 0, s>>>(iota, nnz);
         int bits = 0;
         while (bits < 32 && ((uint32_t)(n - 1) >> bits) != 0) ++bits;
-        e = radix_sort_pairs((const uint32_t *)ci, iota, kout, tmap, nnz, bits, s);
+        e = radix_sort_pairs((const uint32_t *)ci, iota, kout, tmap, nnz, bits, s, &tmp);
     }
     if (e == cudaSuccess) e = expand_rows(rp, n, erow, s);
     if (e == cudaSuccess) {
         k_gather_rows<<<grid_of(nnz), 256, 0, s>>>(erow, tmap, nnz, crow);
         e = cudaGetLastError();
     }
-    cudaFreeAsync(cnt, s);
-    cudaFreeAsync(iota, s);
-    cudaFreeAsync(erow, s);
-    cudaFreeAsync(kout, s);
     return e;
 }
 }  // namespace spt

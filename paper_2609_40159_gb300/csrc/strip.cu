@@ -373,13 +373,13 @@ int stage_grid(int64_t groups)
 
 }  // namespace
 
-cudaError_t strip_sizes(const StripBuild &B, cudaStream_t s)
+cudaError_t strip_sizes(const StripBuild &B, cudaStream_t s, const Scratch *from)
 {
     k_strip_reach<<<warp_grid(B.ng), 256, 0, s>>>(B);
     k_strip_sizes<<<warp_grid(B.ng), 256, 0, s>>>(B);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
-        e = exclusive_scan_i32(B.units, reinterpret_cast<int32_t *>(B.ofs), B.ng, B.total, s);
+        e = exclusive_scan_i32(B.units, reinterpret_cast<int32_t *>(B.ofs), B.ng, B.total, s, from);
     return e;
 }
 

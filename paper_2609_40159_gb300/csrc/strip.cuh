@@ -100,7 +100,7 @@ __host__ __device__ inline int32_t strip_ring(int32_t far, int32_t most)
     return want < kStripRingLeast ? kStripRingLeast : want > most ? most : want;
 }
 // Everything but the blocks, then these (ecode: by entry of the list).
-cudaError_t strip_sizes(const StripBuild &B, cudaStream_t s);
+cudaError_t strip_sizes(const StripBuild &B, cudaStream_t s, const Scratch *from);
 cudaError_t strip_tables(const StripBuild &B, const uint32_t *ofs, unsigned char *blocks, uint16_t *ecode,
                          cudaStream_t s);
 
