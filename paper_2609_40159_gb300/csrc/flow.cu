@@ -19,6 +19,7 @@
 // FP64 3.16 -> 1.07 ms and 20.5 -> 12.8 ms, FP32 2.61 -> 0.68 ms and
 // 19.2 -> 9.1 ms; four right-hand sides on 401^2 (FP32) 2.10 -> 0.25 ms.
 #include <algorithm>
+#include <atomic>
 #include <climits>
 
 #include "flow.cuh"
@@ -565,7 +566,19 @@ template <class T> bool flow_fits(int csize)
 
 }  // namespace
 
-bool flow_cluster_fits(int csize, bool f64) { return f64 ? flow_fits<double>(csize) : flow_fits<float>(csize); }
+// (a property of the device: asked once for each device, type and size)
+bool flow_cluster_fits(int csize, bool f64)
+{
+    static std::atomic<int> known[64][2][5];  // 0: not asked, 1: no, 2: yes
+    int device = -1, l = 0;
+    while ((1 << l) < csize) ++l;
+    const bool keep = cudaGetDevice(&device) == cudaSuccess && device >= 0 && device < 64 && l < 5;
+    const int k = keep ? known[device][f64][l].load() : 0;
+    if (k) return k == 2;
+    const bool fits = f64 ? flow_fits<double>(csize) : flow_fits<float>(csize);
+    if (keep) known[device][f64][l] = fits ? 2 : 1;
+    return fits;
+}
 
 cudaError_t flow_order(const int32_t *ptr, const int32_t *lev, int32_t n, int32_t L, bool trans, int32_t *order,
                        int32_t *iperm, int32_t *counts, cudaStream_t s, const Scratch *from)

@@ -29,13 +29,7 @@
 namespace spt {
 
 // ------------------------------------------------------------ prologue
-__global__ void k_prologue(PlanCtl *ctl)
-{
-    ctl->ticket = 0ull;
-    ctl->progress = 0ull;
-    ctl->epoch = ctl->epoch + 1ull;
-    ctl->abort_flag = 0;
-}
+__global__ void k_prologue(PlanCtl *ctl) { reset_ctl(ctl); }
 
 template <class T>
 cudaError_t launch_prologue(PlanCtl *ctl, cudaStream_t s)
@@ -998,8 +992,7 @@ template <class T>
 cudaError_t solve_block(const Sys<T> &A, const Strips &V, const Rhs<T> &R, int rpw, bool trans,
                         const SyncArgs &sy, int nwarps, cudaStream_t s)
 {
-    cudaError_t e = launch_prologue<T>(sy.ctl, s);
-    if (e == cudaSuccess && rpw == 32) e = strip_stage<T>(A, V, trans, s);
+    cudaError_t e = rpw == 32 && A.n > 0 ? strip_stage<T>(A, V, sy.ctl, trans, s) : launch_prologue<T>(sy.ctl, s);
     if (e != cudaSuccess || A.n <= 0) return e;
     if (rpw == 32) {
         // the columns are independent chains, and a block's chain grows with

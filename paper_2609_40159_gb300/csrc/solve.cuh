@@ -104,6 +104,14 @@ template <auto Kernel> cudaError_t allow_smem(int bytes)
 // All return cudaSuccess or the launch error; T = double or float.
 template <class T>
 cudaError_t launch_prologue(PlanCtl *ctl, cudaStream_t s);
+// The same inside the first kernel of a solve, by one of its threads.
+__device__ __forceinline__ void reset_ctl(PlanCtl *ctl)
+{
+    ctl->ticket = 0ull;
+    ctl->progress = 0ull;
+    ctl->epoch = ctl->epoch + 1ull;
+    ctl->abort_flag = 0;
+}
 
 template <class T>
 cudaError_t solve_level_launch(const Sys<T> &A, const int32_t *perm,

@@ -337,8 +337,9 @@ __device__ void stage_group(const Sys<T> &A, const Strips &V, int64_t g, unsigne
 }
 
 template <class T, bool TR>
-__global__ void __launch_bounds__(32 * kStageWarps) k_strip_stage(Sys<T> A, Strips V)
+__global__ void __launch_bounds__(32 * kStageWarps) k_strip_stage(Sys<T> A, Strips V, PlanCtl *ctl)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) reset_ctl(ctl);
     extern __shared__ __align__(16) unsigned char smraw[];
     const int64_t ng = ((int64_t)A.n + 31) / 32;
     const int64_t nw = (int64_t)gridDim.x * kStageWarps;
@@ -390,15 +391,16 @@ cudaError_t strip_tables(const StripBuild &B, const uint32_t *ofs, unsigned char
     return cudaGetLastError();
 }
 
-template <class T> cudaError_t strip_stage(const Sys<T> &A, const Strips &V, bool trans, cudaStream_t s)
+template <class T>
+cudaError_t strip_stage(const Sys<T> &A, const Strips &V, PlanCtl *ctl, bool trans, cudaStream_t s)
 {
     if (A.n <= 0) return cudaSuccess;
     constexpr int smem = kStageWarps * kStageBytes<T>;
     const int grid = stage_grid(((int64_t)A.n + 31) / 32);
     const cudaError_t e = trans ? allow_smem<k_strip_stage<T, true>>(smem) : allow_smem<k_strip_stage<T, false>>(smem);
     if (e != cudaSuccess) return e;
-    if (trans) k_strip_stage<T, true><<<grid, 32 * kStageWarps, smem, s>>>(A, V);
-    else k_strip_stage<T, false><<<grid, 32 * kStageWarps, smem, s>>>(A, V);
+    if (trans) k_strip_stage<T, true><<<grid, 32 * kStageWarps, smem, s>>>(A, V, ctl);
+    else k_strip_stage<T, false><<<grid, 32 * kStageWarps, smem, s>>>(A, V, ctl);
     return cudaGetLastError();
 }
 
@@ -418,7 +420,7 @@ cudaError_t strip_stage_batch(const BatchMat *mats, const RowChunk *chunks, int6
 }
 
 #define SPT_INST(T)                                                                                   \
-    template cudaError_t strip_stage<T>(const Sys<T> &, const Strips &, bool, cudaStream_t);          \
+    template cudaError_t strip_stage<T>(const Sys<T> &, const Strips &, PlanCtl *, bool, cudaStream_t); \
     template cudaError_t strip_stage_batch<T>(const BatchMat *, const RowChunk *, int64_t, bool,      \
                                               cudaStream_t);
 SPT_INST(double)

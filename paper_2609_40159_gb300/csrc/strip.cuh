@@ -105,8 +105,10 @@ cudaError_t strip_tables(const StripBuild &B, const uint32_t *ofs, unsigned char
                          cudaStream_t s);
 
 // The refresh before a solve: of one system, or of every group of a batch
-// (chunks: (system, 32 * group)).
-template <class T> cudaError_t strip_stage(const Sys<T> &A, const Strips &V, bool trans, cudaStream_t s);
+// (chunks: (system, 32 * group)).  Of a single system: resets the control block
+// for the solve that follows too (small systems wait for the host's launches).
+template <class T>
+cudaError_t strip_stage(const Sys<T> &A, const Strips &V, PlanCtl *ctl, bool trans, cudaStream_t s);
 template <class T>
 cudaError_t strip_stage_batch(const BatchMat *mats, const RowChunk *chunks, int64_t nchunks, bool trans,
                               cudaStream_t s);
