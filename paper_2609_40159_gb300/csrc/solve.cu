@@ -690,20 +690,20 @@ size_t block_smem_bytes(int rpw, int kt, int kc, bool f64)
     return ring * kt * (f64 ? 8 : 4) + ring * 4 + (size_t)kc * 4 + 16;
 }
 // ------------------------------------------------------------- gradient
-// One warp per 32 rows, their nonzeros one per lane: with eight lanes per row
-// half the lanes of a short row idle, and an FP64 multiply-add takes its 19
-// cycles of the SM whatever the lanes do.
+// One warp per `rows` rows (at most 32), their nonzeros one per lane: with eight
+// lanes per row half the lanes of a short row idle, and an FP64 multiply-add
+// takes its 19 cycles of the SM whatever the lanes do.
 // 128^3 Laplacian, FP64, 8 columns: about 135 us (eight lanes per row, one element
 // a load: 261 us; the multiply-adds alone: 127 us).
 template <class T, int V>
 __global__ void __launch_bounds__(256) k_grad_vals(Sys<T> A, const T *__restrict__ gb, const T *__restrict__ x,
-                                                   int64_t ld, int32_t k, T *__restrict__ gv)
+                                                   int64_t ld, int32_t k, int rows, T *__restrict__ gv)
 {
     const int lane = threadIdx.x & 31;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t r0 = gw * 32; r0 < A.n; r0 += nw * 32) {
-        const int nrows = (int)min((int64_t)32, A.n - r0);
+    for (int64_t r0 = gw * rows; r0 < A.n; r0 += nw * rows) {
+        const int nrows = (int)min((int64_t)rows, A.n - r0);
         const int s = ldro(A.rp + r0 + min(lane, nrows));
         const int p0 = __shfl_sync(SPT_FULL_MASK, s, 0), end = ldro(A.rp + r0 + nrows);
         for (int base = p0; base < end; base += 32) {
@@ -714,16 +714,30 @@ __global__ void __launch_bounds__(256) k_grad_vals(Sys<T> A, const T *__restrict
     }
 }
 
+// Rows of a warp: 32, which keeps its lanes busy, but 4 or 8 where the 64 warps
+// that an SM holds then cover the system at once (with 32 a small system's few
+// warps take round after round).  FP64, 32 columns, us with eight lanes per row
+// / 32 / 8 / 4 rows a warp: 1,000 rows 10.3 / 23.3 / 9.2 / 8.4, 4,000 longer
+// ones 12.5 / 40.6 / 14.5 / 10.5, 40,000 24.8 / 18.6 / 14.6 / 22.8; FP32, one
+// column, 1,000,000 rows 31.9 / 16.6 / 20.7 / 37.2.
+static int grad_rows(int32_t n)
+{
+    for (int rows : {4, 8})
+        if ((int64_t)n <= (int64_t)rows * 152 * 64) return rows;
+    return 32;
+}
+
 template <class T>
 cudaError_t grad_vals(const Sys<T> &A, const T *gb, const T *x, int64_t ld, int32_t k, T *gv,
                       cudaStream_t s)
 {
     if (A.n <= 0) return cudaSuccess;
-    const int64_t blocks = std::min<int64_t>(((int64_t)A.n + 255) / 256, 152 * 16);
+    const int rows = grad_rows(A.n);
+    const int64_t blocks = std::min<int64_t>(((int64_t)A.n + 8 * rows - 1) / (8 * rows), 152 * 16);
     const int v = row_vec<T>(gb, x, ld, k);
-    if (v == 4) k_grad_vals<T, 16 / sizeof(T)><<<(int)blocks, 256, 0, s>>>(A, gb, x, ld, k, gv);
-    else if (v == 2) k_grad_vals<T, 2><<<(int)blocks, 256, 0, s>>>(A, gb, x, ld, k, gv);
-    else k_grad_vals<T, 1><<<(int)blocks, 256, 0, s>>>(A, gb, x, ld, k, gv);
+    if (v == 4) k_grad_vals<T, 16 / sizeof(T)><<<(int)blocks, 256, 0, s>>>(A, gb, x, ld, k, rows, gv);
+    else if (v == 2) k_grad_vals<T, 2><<<(int)blocks, 256, 0, s>>>(A, gb, x, ld, k, rows, gv);
+    else k_grad_vals<T, 1><<<(int)blocks, 256, 0, s>>>(A, gb, x, ld, k, rows, gv);
     return cudaGetLastError();
 }
 

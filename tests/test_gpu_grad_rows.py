@@ -48,3 +48,16 @@ def test_grad_rows_batch(dt):
     gv = plan.grad_vals(pack(gb), pack(x)).cpu().numpy()
     for m, A in enumerate(hosts):
         _check(gv[plan.vals_offset[m]:plan.vals_offset[m + 1]], A, gb[m], x[m], dt)
+
+
+@pytest.mark.parametrize("dt", [np.float64, np.float32], ids=["f64", "f32"])
+@pytest.mark.parametrize("n", [3, 5, 38_912, 38_913, 77_824, 77_829])
+def test_grad_rows_of_a_warp(n, dt):
+    """On both sides of the sizes where a warp takes more rows."""
+    import paper_2609_40159_gb300 as P
+    A_h = S.band_random(n, 300, 0, 9, seed=n).astype(dt)
+    plan = P.Plan(P.Matrix.from_host(A_h), mode="syncfree")
+    for k in (1, 3, 4):
+        gb, x = S.rhs(n, k, seed=4, dtype=dt), S.rhs(n, k, seed=5, dtype=dt)
+        gv = plan.grad_vals(torch.as_tensor(gb).cuda(), torch.as_tensor(x).cuda())
+        _check(gv.cpu().numpy(), A_h, gb, x, dt)
