@@ -175,6 +175,7 @@ struct sptrsv_plan_st {
         std::vector<int32_t> rpw, tile, sched;
         bool csc_vals = false;  // some item reads L's values in CSC order
         bool strips = false;    // some item is solved over strips
+        int stage = 0;          // shared memory of a group's refresh
         BatchItem *d_items = nullptr;
         int32_t *d_order = nullptr;
         int32_t nitems = 0;
@@ -581,11 +582,11 @@ void build_strips(sptrsv_plan p, const std::vector<PlanMat *> (&mats)[2], const 
             nnz[d] += M.L.nnz;
         }
     cudaStream_t s = p->h->stream;
-    // scratch: the systems; totals and reaches (read back); then by direction
+    // scratch: the systems; totals, refresh memory and reaches (read back); then by direction
     // and group offsets (copied to the tables), sizes and contents
     char *tmp = nullptr, *tab = nullptr;
     const size_t b_src = sizeof(StripSrc) * all, b_ofs[2] = {4 * ((size_t)ng[0] + 1), 4 * ((size_t)ng[1] + 1)};
-    const size_t b_back = 16 + 4 * all, at_ofs = (b_src + b_back + 15) / 16 * 16;
+    const size_t b_back = 24 + 4 * all, at_ofs = (b_src + b_back + 15) / 16 * 16;
     Scratch scratch(s, from);
     cudaError_t e = scratch.take(&tmp, at_ofs + b_ofs[0] + b_ofs[1] + 8 * (size_t)(ng[0] + ng[1]));
     if (e != cudaSuccess) { cudaGetLastError(); return; }
@@ -594,7 +595,8 @@ void build_strips(sptrsv_plan p, const std::vector<PlanMat *> (&mats)[2], const 
     for (int d = 0; d < 2; ++d) {
         B[d].total = reinterpret_cast<int64_t *>(tmp + b_src) + d;
         B[d].src = reinterpret_cast<StripSrc *>(tmp) + d * nm[0];
-        B[d].far = reinterpret_cast<int32_t *>(tmp + b_src + 16) + d * nm[0];
+        B[d].stage = reinterpret_cast<int32_t *>(tmp + b_src + 16) + d;
+        B[d].far = reinterpret_cast<int32_t *>(tmp + b_src + 24) + d * nm[0];
         B[d].ofs = reinterpret_cast<uint32_t *>(tmp + at_ofs + (d ? b_ofs[0] : 0));
         B[d].units = reinterpret_cast<int32_t *>(u);
         B[d].bits = u + ng[d];
@@ -625,11 +627,12 @@ void build_strips(sptrsv_plan p, const std::vector<PlanMat *> (&mats)[2], const 
         unsigned char *blocks = reinterpret_cast<unsigned char *>(tab) + (d ? 16 * (size_t)total[0] : 0);
         uint32_t *ofs = reinterpret_cast<uint32_t *>(tab + b_blocks + (d ? b_ofs[0] : 0));
         uint16_t *ecode = reinterpret_cast<uint16_t *>(tab + b_blocks + b_ofs[0] + b_ofs[1]) + (d ? nnz[0] : 0);
-        const int32_t *far = reinterpret_cast<const int32_t *>(back.data() + 16) + d * nm[0];
+        const int32_t *far = reinterpret_cast<const int32_t *>(back.data() + 24) + d * nm[0];
+        const int32_t stage = reinterpret_cast<const int32_t *>(back.data() + 16)[d];
         e = strip_tables(B[d], ofs, blocks, ecode, s);
         for (size_t m = 0; m < nm[d] && e == cudaSuccess; ++m)
             mats[d][m]->strips[d] = Strips{blocks, ofs + src[d * nm[0] + m].g0, ecode + src[d * nm[0] + m].e0,
-                                           strip_ring(far[m], B[d].ring_most)};
+                                           strip_ring(far[m], B[d].ring_most), stage};
     }
     if (e != cudaSuccess && tab) {
         for (int d = 0; d < 2; ++d)
@@ -1310,6 +1313,7 @@ sptrsv_status rebuild_items(sptrsv_plan p, int dir)
     std::vector<double> est;
     size_t smem = 16;
     G.csc_vals = G.strips = false;
+    G.stage = 0;
     auto takes_strips = [&](int m) { return p->takes_strips(dir, m); };
     std::vector<PlanMat *> need[2];
     p->strips_to_build(dir, &need[dir]);
@@ -1347,6 +1351,7 @@ sptrsv_status rebuild_items(sptrsv_plan p, int dir)
             I.rpw = I.sched == kSchedLevel ? 32 : G.rpw[m] == 32 && !one_lane ? 16 : G.rpw[m];
             if (I.sched == kSchedInOrder && I.rpw == 32) {
                 G.strips = true;
+                G.stage = std::max(G.stage, (int)M.strips[dir].stage);
                 I.nw = kBatchWarps;
                 smem = std::max(smem, strip_smem(M.strips[dir].ring, I.KT, f64, kBatchWarps));
             } else {
@@ -1692,8 +1697,8 @@ sptrsv_status batch_solve_impl(sptrsv_plan p, const void *b, void *x, bool trans
                                    : batch_csc_values<float>(p->d_mats, p->d_ctiles, p->n_ctiles, p->h->stream);
     if (e == cudaSuccess && G.strips)
         e = p->dtype == SPTRSV_F64
-                ? strip_stage_batch<double>(p->d_mats, p->d_gchunks, p->n_gchunks, trans, p->h->stream)
-                : strip_stage_batch<float>(p->d_mats, p->d_gchunks, p->n_gchunks, trans, p->h->stream);
+                ? strip_stage_batch<double>(p->d_mats, p->d_gchunks, p->n_gchunks, G.stage, trans, p->h->stream)
+                : strip_stage_batch<float>(p->d_mats, p->d_gchunks, p->n_gchunks, G.stage, trans, p->h->stream);
     if (e != cudaSuccess) return from_cuda(e);
     if (p->dtype == SPTRSV_F64)
         e = batch_solve<double>(p->d_mats, G.d_items, G.nitems, G.d_order, (const double *)b, (double *)x,

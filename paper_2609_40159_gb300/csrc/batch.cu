@@ -269,8 +269,8 @@ int batch_grid(size_t smem, const DeviceInfo &di)
     cudaFuncSetAttribute(k_batch<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_batch<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_batch<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    strip_stage_batch<float>(nullptr, nullptr, 0, false, nullptr);
-    strip_stage_batch<double>(nullptr, nullptr, 0, false, nullptr);
+    strip_stage_batch<float>(nullptr, nullptr, 0, 0, false, nullptr);
+    strip_stage_batch<double>(nullptr, nullptr, 0, 0, false, nullptr);
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch<float, false>, kBatchThreads, smem);
     if (per_sm < 1) per_sm = 1;

@@ -86,6 +86,7 @@ struct Strips {
     const uint32_t *ofs;    // start of every group's block, in units of 16 bytes; the end
     const uint16_t *ecode;  // by entry: where its value goes (strip.cu)
     int32_t ring;           // rows of a column's ring of solutions
+    int32_t stage;          // shared memory that the refresh of a group takes, at most
 };
 
 // ---------------------------------------------------------------- launchers

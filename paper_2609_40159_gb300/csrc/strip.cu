@@ -14,11 +14,18 @@ namespace {
 constexpr uint16_t kToTri = 0x8000, kToDiag = 0x4000, kNowhere = 0x2000, kScaled = 0x1000;
 
 constexpr int kStageWarps = 4;
+constexpr int kStageEntries = 12;  // (11 a row in the mean fit a group in one go)
 constexpr int kTri = 36;       // row stride of a triangle in shared memory
 constexpr float kMaxInverse = 16.0f;
 constexpr int kMaxSteps = 8;   // FP32: longer schedules become an inverse
-// Quads of a group that are put together: of dependencies, and of steps.
-template <class T> constexpr int kMaxQuads = (kStripNear + kStripOld) / 4 + (sizeof(T) == 8 ? 8 : (kMaxSteps + 3) / 4);
+// Shared memory that the refresh of a group takes (values of w bytes): the
+// diagonals, the quads put together (of dependencies, and of steps), and the
+// triangle where it becomes an inverse.
+__host__ __device__ __forceinline__ int stage_bytes(const StripBits &h, int w)
+{
+    const int inv = h.kind == kTriInverse;
+    return 32 * w + 128 * w * (h.staged() + (inv ? 0 : h.tri_quads())) + (inv ? 32 * kTri * w : 0);
+}
 
 // What a row's entries are to its group: dependencies of the group itself
 // (mask), of the previous group (nb), older ones (na); entries from `ptail` on
@@ -129,7 +136,10 @@ __global__ void __launch_bounds__(256) k_strip_sizes(StripBuild B)
         const uint32_t kind = steps == 0 ? kTriNone : !B.f64 && steps > kMaxSteps ? kTriInverse : kTriSteps;
         if (lane == 0) {
             B.bits[g] = strip_bits(na, nb, kind, steps, tail, far > ring - 32);
-            B.units[g] = StripBits(B.bits[g]).bytes(B.f64 ? 8 : 4) / 16;
+            const StripBits h(B.bits[g]);
+            B.units[g] = h.bytes(B.f64 ? 8 : 4) / 16;
+            const int need = stage_bytes(h, B.f64 ? 8 : 4);
+            if (need > *B.stage) atomicMax(B.stage, need);
         }
     }
 }
@@ -243,24 +253,55 @@ __device__ __forceinline__ float invert_triangle(float *c, int lane)
     return big;
 }
 
-template <class T>
-constexpr int kStageBytes = kMaxQuads<T> * 128 * (int)sizeof(T) + 32 * (int)sizeof(T) + (sizeof(T) == 4 ? 32 * kTri * 4 : 0);
+// Where a group's block and entries are.  Loaded while the group before is
+// staged: what a group's entries wait for would otherwise be three loads from
+// memory one after another.
+struct StageAt {
+    unsigned char *blk;
+    uint32_t bits;
+    int p0, p1;
+    __device__ __forceinline__ StageAt() : blk(nullptr), bits(0u), p0(0), p1(0) {}
+    template <class T> __device__ __forceinline__ StageAt(const Sys<T> &A, const Strips &V, int g, bool trans)
+    {
+        blk = V.blocks + (size_t)ldro(V.ofs + g) * 16u;
+        bits = *reinterpret_cast<const uint32_t *>(blk);
+        const int base = g * 32, rows = min(32, A.n - base), lo = trans ? A.n - base - rows : base;
+        const int32_t *ptr = trans ? A.cp : A.rp;
+        p0 = ldro(ptr + lo);
+        p1 = ldro(ptr + lo + rows);
+    }
+};
+
+// The groups of a warp: a block takes consecutive ones, its warps in turn, as
+// neighbours share the lines of the tables and, transposed, of the values that
+// they gather.
+struct StageShare {
+    int64_t first, end;
+    __device__ __forceinline__ explicit StageShare(int64_t groups)
+    {
+        const int64_t per = (groups + (int64_t)gridDim.x * kStageWarps - 1) / ((int64_t)gridDim.x * kStageWarps);
+        const int64_t start = blockIdx.x * per * kStageWarps;
+        first = start + (threadIdx.x >> 5);
+        end = min(groups, start + per * kStageWarps);
+    }
+};
 
 // One group's values into its block, by one warp.  The entries of the group's
 // rows are contiguous (CSR forward, CSC transpose), so everything is read and
 // written along lanes; the quads are put together in shared memory.
 template <class T, bool TR>
-__device__ void stage_group(const Sys<T> &A, const Strips &V, int64_t g, unsigned char *raw)
+__device__ __forceinline__ void stage_group(const Sys<T> &A, const Strips &V, int g, const StageAt &at,
+                                            unsigned char *raw)
 {
     constexpr int HV = 16 / (int)sizeof(T);  // values of 16 bytes
     const int lane = threadIdx.x & 31;
-    T *quads = reinterpret_cast<T *>(raw);  // as in the block: FP32 [quad][row][4], FP64 [quad][half][row][2]
-    T *diag = quads + kMaxQuads<T> * 128;
-    float *tri = reinterpret_cast<float *>(diag + 32);
-    unsigned char *blk = V.blocks + (size_t)ldro(V.ofs + g) * 16u;
-    const StripBits h(*reinterpret_cast<const uint32_t *>(blk));
-    const int base = (int)(g * 32), rows = min(32, A.n - base);
+    T *diag = reinterpret_cast<T *>(raw);
+    T *quads = diag + 32;  // as in the block: FP32 [quad][row][4], FP64 [quad][half][row][2]
+    unsigned char *blk = at.blk;
+    const StripBits h(at.bits);
+    const int rows = min(32, A.n - g * 32);
     const int staged = h.staged(), qv = staged + (h.kind == kTriInverse ? 0 : h.tri_quads());
+    float *tri = reinterpret_cast<float *>(quads + qv * 128);
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     float4 *q4 = reinterpret_cast<float4 *>(quads);
     constexpr int P = 4 / HV;  // 16-byte planes of a quad
@@ -272,33 +313,32 @@ __device__ void stage_group(const Sys<T> &A, const Strips &V, int64_t g, unsigne
             for (int q = 0; q < 32; q += 4) *reinterpret_cast<float4 *>(tri + lane * kTri + q) = zero;
     }
     __syncwarp();
-    // rows [lo, lo + rows) of the matrix
-    const int lo = TR ? A.n - base - rows : base;
-    const int32_t *ptr = TR ? A.cp : A.rp;
-    const int p0 = ldro(ptr + lo), p1 = ldro(ptr + lo + rows);
-    // eight entries a lane at a time: the loads of all are in flight together
+    // several entries a lane at a time: the loads of all are in flight together
     // (one at a time: 2.4x)
-    for (int pa = p0 + lane; pa - lane < p1; pa += 256) {
-        unsigned c[8];
-        T v[8];
+    const int p1 = at.p1;
+    for (int pa = at.p0 + lane; pa - lane < p1; pa += 32 * kStageEntries) {
+        unsigned c[kStageEntries];
+        T v[kStageEntries];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
+        for (int u = 0; u < kStageEntries; ++u) {
             const int p = pa + 32 * u;
             c[u] = p < p1 ? ldro(V.ecode + p) : kNowhere;
+            v[u] = p < p1 ? entry_val<T, TR>(A, p) : T(0);
+        }
+        // (all of them: left to itself the compiler moves each value's load to its
+        // store, behind the store before)
+#pragma unroll
+        for (int u = 0; u < kStageEntries; ++u) {
+            consume((int)c[u]);
+            consume(v[u]);
         }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = c[u] & kNowhere ? T(0) : entry_val<T, TR>(A, pa + 32 * u);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            if (c[u] & kNowhere) continue;
-            if (c[u] & kToTri) {
-                tri[((c[u] >> 5) & 31) * kTri + (c[u] & 31)] = (float)v[u];
-            } else if (c[u] & kToDiag) {
-                diag[c[u] & 31] = v[u];
-            } else {
-                const int slot = c[u] & 127, row = (c[u] >> 7) & 31;
-                quads[((slot / HV) * 32 + row) * HV + slot % HV] = v[u];
-            }
+        for (int u = 0; u < kStageEntries; ++u) {
+            const int row = (c[u] & (kToTri | kToDiag)) ? (c[u] >> 5) & 31 : (c[u] >> 7) & 31, slot = c[u] & 127;
+            T *to = quads + ((slot / HV) * 32 + row) * HV + slot % HV;
+            if (sizeof(T) == 4) to = c[u] & kToTri ? reinterpret_cast<T *>(tri + row * kTri + (c[u] & 31)) : to;
+            to = c[u] & kToDiag ? diag + (c[u] & 31) : to;
+            if (!(c[u] & kNowhere)) *to = v[u];
         }
     }
     __syncwarp();
@@ -341,28 +381,48 @@ __global__ void __launch_bounds__(32 * kStageWarps) k_strip_stage(Sys<T> A, Stri
 {
     if (blockIdx.x == 0 && threadIdx.x == 0) reset_ctl(ctl);
     extern __shared__ __align__(16) unsigned char smraw[];
+    unsigned char *raw = smraw + (threadIdx.x >> 5) * V.stage;
     const int64_t ng = ((int64_t)A.n + 31) / 32;
-    const int64_t nw = (int64_t)gridDim.x * kStageWarps;
-    for (int64_t g = (int64_t)blockIdx.x * kStageWarps + (threadIdx.x >> 5); g < ng; g += nw)
-        stage_group<T, TR>(A, V, g, smraw + (threadIdx.x >> 5) * kStageBytes<T>);
+    const StageShare sh(ng);
+    StageAt next;
+    if (sh.first < sh.end) next = StageAt(A, V, (int)sh.first, TR);
+    for (int64_t g = sh.first; g < sh.end; g += kStageWarps) {
+        const StageAt at = next;
+        if (g + kStageWarps < sh.end) next = StageAt(A, V, (int)g + kStageWarps, TR);
+        stage_group<T, TR>(A, V, (int)g, at, raw);
+    }
 }
 
 template <class T, bool TR>
 __global__ void __launch_bounds__(32 * kStageWarps)
-k_strip_stage_batch(const BatchMat *__restrict__ mats, const RowChunk *__restrict__ chunks, int64_t nchunks)
+k_strip_stage_batch(const BatchMat *__restrict__ mats, const RowChunk *__restrict__ chunks, int64_t nchunks, int stage)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
-    const int64_t nw = (int64_t)gridDim.x * kStageWarps;
-    for (int64_t c = (int64_t)blockIdx.x * kStageWarps + (threadIdx.x >> 5); c < nchunks; c += nw) {
-        const RowChunk ch = chunks[c];
-        const BatchMat &M = mats[ch.mat];
-        if (M.strips[TR ? 1 : 0].blocks == nullptr) continue;
+    unsigned char *raw = smraw + (threadIdx.x >> 5) * stage;
+    const StageShare sh(nchunks);
+    auto sys = [&](const BatchMat &M) {
         Sys<T> A{};
         A.n = M.n;
         A.nnz = M.nnz;
         A.rp = M.rp; A.v = (const T *)M.v;
         A.cp = M.cp; A.tmap = M.tmap;
-        stage_group<T, TR>(A, M.strips[TR ? 1 : 0], ch.r0 >> 5, smraw + (threadIdx.x >> 5) * kStageBytes<T>);
+        return A;
+    };
+    auto look = [&](int64_t c) {
+        const RowChunk ch = chunks[c];
+        const BatchMat &M = mats[ch.mat];
+        const Strips V = M.strips[TR ? 1 : 0];
+        return V.blocks ? StageAt(sys(M), V, ch.r0 >> 5, TR) : StageAt();
+    };
+    StageAt next;
+    if (sh.first < sh.end) next = look(sh.first);
+    for (int64_t c = sh.first; c < sh.end; c += kStageWarps) {
+        const StageAt at = next;
+        if (c + kStageWarps < sh.end) next = look(c + kStageWarps);
+        if (at.blk == nullptr) continue;
+        const RowChunk ch = chunks[c];
+        const BatchMat &M = mats[ch.mat];
+        stage_group<T, TR>(sys(M), M.strips[TR ? 1 : 0], ch.r0 >> 5, at, raw);
     }
 }
 
@@ -395,9 +455,9 @@ template <class T>
 cudaError_t strip_stage(const Sys<T> &A, const Strips &V, PlanCtl *ctl, bool trans, cudaStream_t s)
 {
     if (A.n <= 0) return cudaSuccess;
-    constexpr int smem = kStageWarps * kStageBytes<T>;
+    const int smem = kStageWarps * V.stage, most = (int)kBlockSmemBudget;
     const int grid = stage_grid(((int64_t)A.n + 31) / 32);
-    const cudaError_t e = trans ? allow_smem<k_strip_stage<T, true>>(smem) : allow_smem<k_strip_stage<T, false>>(smem);
+    const cudaError_t e = trans ? allow_smem<k_strip_stage<T, true>>(most) : allow_smem<k_strip_stage<T, false>>(most);
     if (e != cudaSuccess) return e;
     if (trans) k_strip_stage<T, true><<<grid, 32 * kStageWarps, smem, s>>>(A, V, ctl);
     else k_strip_stage<T, false><<<grid, 32 * kStageWarps, smem, s>>>(A, V, ctl);
@@ -405,23 +465,23 @@ cudaError_t strip_stage(const Sys<T> &A, const Strips &V, PlanCtl *ctl, bool tra
 }
 
 template <class T>
-cudaError_t strip_stage_batch(const BatchMat *mats, const RowChunk *chunks, int64_t nchunks, bool trans,
+cudaError_t strip_stage_batch(const BatchMat *mats, const RowChunk *chunks, int64_t nchunks, int stage, bool trans,
                               cudaStream_t s)
 {
-    constexpr int smem = kStageWarps * kStageBytes<T>;
+    const int smem = kStageWarps * stage, most = (int)kBlockSmemBudget;
     // (both, also without chunks: a plan calls this once outside any capture)
-    cudaError_t e = allow_smem<k_strip_stage_batch<T, true>>(smem);
-    if (e == cudaSuccess) e = allow_smem<k_strip_stage_batch<T, false>>(smem);
+    cudaError_t e = allow_smem<k_strip_stage_batch<T, true>>(most);
+    if (e == cudaSuccess) e = allow_smem<k_strip_stage_batch<T, false>>(most);
     if (e != cudaSuccess || nchunks <= 0) return e;
     const int grid = stage_grid(nchunks);
-    if (trans) k_strip_stage_batch<T, true><<<grid, 32 * kStageWarps, smem, s>>>(mats, chunks, nchunks);
-    else k_strip_stage_batch<T, false><<<grid, 32 * kStageWarps, smem, s>>>(mats, chunks, nchunks);
+    if (trans) k_strip_stage_batch<T, true><<<grid, 32 * kStageWarps, smem, s>>>(mats, chunks, nchunks, stage);
+    else k_strip_stage_batch<T, false><<<grid, 32 * kStageWarps, smem, s>>>(mats, chunks, nchunks, stage);
     return cudaGetLastError();
 }
 
 #define SPT_INST(T)                                                                                   \
     template cudaError_t strip_stage<T>(const Sys<T> &, const Strips &, PlanCtl *, bool, cudaStream_t); \
-    template cudaError_t strip_stage_batch<T>(const BatchMat *, const RowChunk *, int64_t, bool,      \
+    template cudaError_t strip_stage_batch<T>(const BatchMat *, const RowChunk *, int64_t, int, bool, \
                                               cudaStream_t);
 SPT_INST(double)
 SPT_INST(float)

@@ -93,6 +93,7 @@ struct StripBuild {
     int32_t *units;       // by group: size of its block (16 bytes)
     uint32_t *ofs;        // the sizes' prefix sums (ng + 1)
     int64_t *total;
+    int32_t *stage;       // the most shared memory that the refresh of a group takes
 };
 __host__ __device__ inline int32_t strip_ring(int32_t far, int32_t most)
 {
@@ -105,12 +106,12 @@ cudaError_t strip_tables(const StripBuild &B, const uint32_t *ofs, unsigned char
                          cudaStream_t s);
 
 // The refresh before a solve: of one system, or of every group of a batch
-// (chunks: (system, 32 * group)).  Of a single system: resets the control block
+// (chunks: (system, 32 * group); stage: the most of its systems' Strips).  Of a single system: resets the control block
 // for the solve that follows too (small systems wait for the host's launches).
 template <class T>
 cudaError_t strip_stage(const Sys<T> &A, const Strips &V, PlanCtl *ctl, bool trans, cudaStream_t s);
 template <class T>
-cudaError_t strip_stage_batch(const BatchMat *mats, const RowChunk *chunks, int64_t nchunks, bool trans,
+cudaError_t strip_stage_batch(const BatchMat *mats, const RowChunk *chunks, int64_t nchunks, int stage, bool trans,
                               cudaStream_t s);
 
 // The system again, every entry on its own: with an infinite or NaN solution
