@@ -172,7 +172,7 @@ struct sptrsv_plan_st {
     // rows per warp and rhs columns per work item, the items (system, rhs
     // column tile, geometry), their launch order, shared memory and grid
     struct Geom {
-        std::vector<int32_t> rpw, tile, sched;
+        std::vector<int32_t> rpw, tile, sched;  // (tile 0: automatic)
         bool csc_vals = false;  // some item reads L's values in CSC order
         bool strips = false;    // some item is solved over strips
         int stage = 0;          // shared memory of a group's refresh
@@ -183,6 +183,16 @@ struct sptrsv_plan_st {
         int grid = 0;
     } geo[2];
     int32_t max_items = 0;
+    // Columns an item: the plan's option, else two, four level by level in FP32
+    // (on 256 training systems of 1,000-40,000 rows over strips, FP32, 3.43 /
+    // 3.03 / 3.40 ms a step with 1 / 2 / 4; on 32 small FP64 ones 0.41 / 0.42 /
+    // 0.63 ms; 64 systems level by level, forward, FP32 0.62 / 0.60 ms with 2 /
+    // 4, FP64 2.9 / 5.3 ms)
+    int tile_of(int d, size_t m) const
+    {
+        if (geo[d].tile[m]) return geo[d].tile[m];
+        return geo[d].sched[m] == kSchedLevel && dtype == SPTRSV_F32 ? 4 : 2;
+    }
     bool takes_strips(int d, size_t m) const
     {
         return geo[d].rpw[m] == 32 && geo[d].sched[m] == kSchedInOrder && mats[m].L.n > 0;
@@ -1155,7 +1165,7 @@ extern "C" sptrsv_status sptrsv_plan_info(sptrsv_plan p, int32_t *nlevels, int32
     }
     if (mode) *mode = p->batched ? SPTRSV_MODE_BLOCK : p->mode;
     if (rows_per_warp) *rows_per_warp = p->batched ? (p->geo[0].rpw.empty() ? 32 : p->geo[0].rpw[0]) : p->rpw;
-    if (rhs_tile) *rhs_tile = p->batched ? (p->geo[0].tile.empty() ? 4 : p->geo[0].tile[0]) : p->kt;
+    if (rhs_tile) *rhs_tile = p->batched ? (p->geo[0].tile.empty() ? 4 : p->tile_of(0, 0)) : p->kt;
     return SPTRSV_OK;
 }
 
@@ -1336,7 +1346,7 @@ sptrsv_status rebuild_items(sptrsv_plan p, int dir)
     for (int m = 0; m < nmat; ++m) {
         PlanMat &M = p->mats[m];
         const int k = p->h_mats[m].k;
-        int tile = G.tile[m];
+        int tile = p->tile_of(dir, (size_t)m);
         // one lane per row, over the strips
         const bool one_lane = G.rpw[m] == 32 && (!takes_strips(m) || M.strips[dir].blocks || (dir == 1 && !p->have_csc));
         G.csc_vals = G.csc_vals || G.sched[m] == kSchedLevel || !one_lane;
@@ -1538,10 +1548,7 @@ extern "C" sptrsv_status sptrsv_batch_plan_create(sptrsv_handle h, int32_t nmat,
     p->h_mats.resize((size_t)nmat);
     for (int d = 0; d < 2; ++d) {
         p->geo[d].rpw.assign((size_t)nmat, 32);
-        // (two columns an item: on 256 training systems of 1,000-40,000 rows,
-        // FP32, 3.43 / 3.03 / 3.40 ms a step with 1 / 2 / 4; on 32 small FP64
-        // ones 0.41 / 0.42 / 0.63 ms)
-        p->geo[d].tile.assign((size_t)nmat, 2);
+        p->geo[d].tile.assign((size_t)nmat, 0);
         p->geo[d].sched.assign((size_t)nmat, kSchedInOrder);
     }
     int64_t ktot = 0;
