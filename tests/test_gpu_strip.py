@@ -155,3 +155,32 @@ def test_strip_bounded_wait(trans):
     ref = (oracle.solve_transpose if trans else oracle.solve)(A_h, b_h)
     assert relerr(run(b).cpu().numpy(), ref) <= 1e-12
     assert h.status() == 0
+
+
+def test_strip_refresh_takes_several_groups_a_warp():
+    """More groups than the refresh has warps (2.49M rows): a warp goes from
+    group to group, in a single system and across the systems of a batch, of
+    which some have no strips."""
+    import paper_2609_40159_gb300 as P
+    dt = np.float32
+    A_h = S.band_random(2_600_003, 40, 0, 4, seed=3).astype(dt)
+    A, W_h = P.Matrix.from_host(A_h), widened(A_h)
+    b_h = S.rhs(A_h.n, 1, seed=1, dtype=dt)
+    refs = oracle.solve(W_h, b_h), oracle.solve_transpose(W_h, b_h)
+    b = torch.as_tensor(b_h).cuda()
+    plan = P.Plan(A, mode="block", rows_per_warp=32, transpose=True)
+    assert relerr(plan.solve(b).cpu().numpy(), refs[0]) <= TOL[dt]
+    assert relerr(plan.solve_transpose(b).cpu().numpy(), refs[1]) <= TOL[dt]
+    small = S.band_random(1000, 30, 0, 8, seed=4).astype(dt)
+    s_h = S.rhs(small.n, 1, seed=2, dtype=dt)
+    mats, rpw = [], []
+    for m in range(5):
+        mats += [P.Matrix.from_host(small)]
+        rpw += [32 if m % 2 else 16]
+    plan = P.BatchPlan([*mats, A, *mats], nrhs=[1] * 11, rows_per_warp=[*rpw, 32, *rpw], transpose=True)
+    packed = torch.as_tensor(np.concatenate([*[s_h.reshape(-1)] * 5, b_h.reshape(-1), *[s_h.reshape(-1)] * 5])).cuda()
+    for run, ref, big in ((plan.solve, oracle.solve, refs[0]), (plan.solve_transpose, oracle.solve_transpose, refs[1])):
+        x, want = run(packed), ref(widened(small), s_h)
+        for m in range(11):
+            assert relerr(plan.unpack(x, m).cpu().numpy(), big if m == 5 else want) <= TOL[dt], m
+    assert P.handle().status() == 0
