@@ -298,28 +298,54 @@ class Plan:
                              "with unit column stride")
         return b
 
+    @staticmethod
+    def _like(b, x):
+        """(b with x's leading dimension, that dimension): the library takes
+        one for both, so b itself or a copy.  x must hold as many columns."""
+        ld = x.stride(0)
+        if x.shape[1] < b.shape[1]:
+            raise ValueError("the output has fewer columns than the right-hand side")
+        if b.stride(0) == ld or b.shape[0] <= 1:
+            return b, b.stride(0)
+        if min(b.stride(0), ld) < b.shape[1]:
+            raise ValueError("the rows of a block must not overlap")
+        room = torch.empty_strided(b.shape, (ld, 1), dtype=b.dtype, device=b.device)
+        return room.copy_(b), ld
+
     def solve(self, b: torch.Tensor, out: torch.Tensor | None = None) -> torch.Tensor:
         squeeze = b.dim() == 1
         b2 = self._rhs(b, self.A.n, self.A.dtype)
-        x = out if out is not None else torch.empty(self.A.n, b2.shape[1], dtype=b2.dtype, device=b2.device)
-        x2 = self._rhs(x, self.A.n, self.A.dtype)
-        L.check(L.lib().sptrsv_solve(self.p, _ptr(b2), _ptr(x2), b2.shape[1], b2.stride(0)),
-                "sptrsv_solve")
+        k, ld = b2.shape[1], b2.stride(0)
+        if out is None:
+            x = x2 = torch.empty(self.A.n, k, dtype=b2.dtype, device=b2.device)
+        else:
+            x, x2 = out, self._rhs(out, self.A.n, self.A.dtype)
+        if out is not None or ld != k:
+            b2, ld = self._like(b2, x2)
+        L.check(L.lib().sptrsv_solve(self.p, _ptr(b2), _ptr(x2), k, ld), "sptrsv_solve")
         return x.view(-1) if squeeze and out is None else x
 
     def solve_transpose(self, gx: torch.Tensor, out: torch.Tensor | None = None) -> torch.Tensor:
         squeeze = gx.dim() == 1
         g2 = self._rhs(gx, self.A.n, self.A.dtype)
-        gb = out if out is not None else torch.empty(self.A.n, g2.shape[1], dtype=g2.dtype, device=g2.device)
-        L.check(L.lib().sptrsv_solve_transpose(self.p, _ptr(g2), _ptr(gb), g2.shape[1], g2.stride(0)),
-                "sptrsv_solve_transpose")
+        k, ld = g2.shape[1], g2.stride(0)
+        if out is None:
+            gb = gb2 = torch.empty(self.A.n, k, dtype=g2.dtype, device=g2.device)
+        else:
+            gb, gb2 = out, self._rhs(out, self.A.n, self.A.dtype)
+        if out is not None or ld != k:
+            g2, ld = self._like(g2, gb2)
+        L.check(L.lib().sptrsv_solve_transpose(self.p, _ptr(g2), _ptr(gb2), k, ld), "sptrsv_solve_transpose")
         return gb.view(-1) if squeeze and out is None else gb
 
     def grad_vals(self, gb: torch.Tensor, x: torch.Tensor, out: torch.Tensor | None = None):
         gb2 = self._rhs(gb, self.A.n, self.A.dtype)
         x2 = self._rhs(x, self.A.n, self.A.dtype)
+        ld = gb2.stride(0)
+        if gb2.shape != x2.shape or ld != x2.stride(0):
+            gb2, ld = self._like(gb2, x2)
         gv = out if out is not None else torch.empty(self.A.nnz, dtype=self.A.dtype, device=gb2.device)
-        L.check(L.lib().sptrsv_grad_vals(self.p, _ptr(gb2), _ptr(x2), gb2.shape[1], gb2.stride(0),
+        L.check(L.lib().sptrsv_grad_vals(self.p, _ptr(gb2), _ptr(x2), gb2.shape[1], ld,
                                          _ptr(gv)), "sptrsv_grad_vals")
         return gv
 
@@ -327,8 +353,8 @@ class Plan:
         squeeze = gbp.dim() == 1
         g2 = self._rhs(gbp, self.A.n, self.A.dtype)
         gb = out if out is not None else torch.empty_like(g2)
-        L.check(L.lib().sptrsv_tt_apply(self.p, _ptr(g2), _ptr(gb), g2.shape[1], g2.stride(0)),
-                "sptrsv_tt_apply")
+        g2, ld = self._like(g2, self._rhs(gb, self.A.n, self.A.dtype))
+        L.check(L.lib().sptrsv_tt_apply(self.p, _ptr(g2), _ptr(gb), g2.shape[1], ld), "sptrsv_tt_apply")
         return gb.view(-1) if squeeze and out is None else gb
 
     def __del__(self):
