@@ -410,14 +410,15 @@ k_flow(Sys<T> A, FlowSched F, Rhs<T> R, int32_t withhold, Waiter w)
             }
             for (int o = lpr >> 1; o > 0; o >>= 1) acc += shfl_xor(acc, o);
         }
-        if (!ok) break;  // (what is left are the barriers, which the other warps count on)
         const T xi = (bv - acc) * rinv;
-        if (anythere) {
-            if (there) slot_store<true>(other, xi, me.code);
-            if (anymore)
-                for (unsigned m = mask; m; m &= m - 1) slot_store<true>(map_rank(own, __ffs(m) - 1), xi, me.code);
+        if (ok) {  // (a break here instead costs 1 % of every solve)
+            if (anythere) {
+                if (there) slot_store<true>(other, xi, me.code);
+                if (anymore)
+                    for (unsigned m = mask; m; m &= m - 1) slot_store<true>(map_rank(own, __ffs(m) - 1), xi, me.code);
+            }
+            if (here) slot_store<false>(own, xi, me.code);
         }
-        if (here) slot_store<false>(own, xi, me.code);
         if (lead) x[(int64_t)me.row * R.ld] = xi;
         __syncwarp();
     }
