@@ -84,21 +84,27 @@ typedef enum {
     SPTRSV_MODE_LEVEL_LAUNCH = 1,
     /* Level-set solve in ONE persistent launch: warps take row groups in
      * level order and wait on a grid-wide progress counter for the previous
-     * level instead of a launch boundary.                                    */
+     * level instead of a launch boundary.  With 32 rows per warp: one lane
+     * per row and column, each waiting for the solutions it needs.           */
     SPTRSV_MODE_LEVEL_PERSISTENT = 2,
     /* Synchronisation-free solve: row groups taken in row order, each row
      * waits on its own predecessors' ready flags (acquire/release).          */
     SPTRSV_MODE_SYNCFREE = 3,
-    /* Synchronisation-free solve inside one thread block: flags and recent
-     * solution values live in shared memory; for deep, narrow systems where
-     * the cross-SM flag round trip would dominate.                           */
+    /* Solve inside one thread block: recent solutions live in shared memory;
+     * for deep, narrow systems where the cross-SM flag round trip would
+     * dominate.  With 32 rows per warp: groups of 32 rows in order, over
+     * tables ("strips") that the plan builds and every solve refreshes with
+     * L's values; rhs_tile is not used then.                                 */
     SPTRSV_MODE_BLOCK = 4,
     /* Hybrid of the level-set and synchronisation-free schedules (Section 7,
      * related work): rows in level order as in LEVEL_PERSISTENT; a thick
      * level waits for every earlier level, a maximal run of consecutive thin
      * levels (fewer rows than the plan's thin_rows) waits once for the rows
      * before the run, and inside the run each row waits only for its own
-     * predecessors' ready flags.                                             */
+     * predecessors' ready flags.  With the automatic threshold (every level
+     * thin) and grid, one thread-block cluster per right-hand side runs the
+     * schedule over tables that the plan builds; rows_per_warp and rhs_tile
+     * are not used then.                                                     */
     SPTRSV_MODE_HYBRID = 5
 } sptrsv_mode;
 
@@ -107,9 +113,10 @@ typedef struct {
     int32_t rows_per_warp;   /* 1,2,4,8,16,32 (lanes per row = 32/rows_per_warp); 0 = auto */
     int32_t rhs_tile;        /* right-hand sides per pass: 1,2,4,8,16; 0 = auto.
                                 Block mode and batched plans: columns per
-                                thread block (1,2,4,8; at most 4 with 32
-                                rows per warp); wider right-hand sides run
-                                as independent column tiles                */
+                                thread block (1,2,4,8; with 32 rows per
+                                warp at most 4, single systems one while
+                                there is an SM for each); wider right-hand
+                                sides run as independent column tiles      */
     int32_t build_transpose; /* non-zero: prepare sptrsv_solve_transpose / grad  */
     int64_t wait_limit_us;   /* longest a device wait may take before the solve
                                 gives up with SPTRSV_ETIMEOUT (microseconds);

@@ -77,7 +77,7 @@ int default_rpw(int32_t n, int64_t nnz, int64_t long_rows = 0)
 }
 
 // The same for block-local solves, which stage up to 16 dependencies a row on
-// the previous group and 16 older ones: one lane per row for longer rows too.
+// the previous group and 28 older ones: one lane per row for longer rows too.
 int block_rpw(int32_t n, int64_t nnz, int64_t long_rows = 0)
 {
     const int r = default_rpw(n, nnz, long_rows);

@@ -23,7 +23,10 @@ struct FlowLane {
 };
 
 // Schedule of one direction.  Slot g * 32 + l belongs to lane l of group g;
-// the groups are sorted by block of the cluster.
+// the groups are sorted by block of the cluster.  A slot takes 60 bytes (FP64
+// 80) and an entry 4 more; a row of up to 4 entries has one slot, of up to 16
+// four, of up to 64 sixteen, a longer one 32, and the last group of a level and
+// class is filled up to 32 slots.
 struct FlowSched {
     const FlowLane *lanes;
     const uint4 *codes;    // of the lane's first four entries

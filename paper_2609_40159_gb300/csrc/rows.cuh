@@ -1,6 +1,7 @@
 // Row views of a system for the solve kernels: the forward solve reads L by
-// rows (CSR), the transpose solve reads L by columns (CSC, values gathered
-// into CSC order before the solve).
+// rows (CSR), the transpose solve reads L by columns (CSC; the values from a
+// copy gathered into CSC order before the solve, or through the map to L's
+// own: entry_val).
 #pragma once
 
 #include "solve.cuh"
@@ -102,26 +103,6 @@ template <class T> __host__ __device__ __forceinline__ int row_vec(const T *a, c
     int v = 16 / (int)sizeof(T);
     while (v > 1 && bits % ((size_t)v * sizeof(T)) != 0) v >>= 1;
     return v;
-}
-
-// Prefetch into L2 the first line of a row's entries (indices and values).
-__device__ __forceinline__ void prefetch_l2(const void *p)
-{
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-
-template <class T, bool TR>
-__device__ __forceinline__ void prefetch_row(const Sys<T> &A, int i)
-{
-    if (!TR) {
-        const int a = ldro(A.rp + i);
-        prefetch_l2(A.ci + a);
-        prefetch_l2(A.v + a);
-    } else {
-        const int a = ldro(A.cp + i);
-        prefetch_l2(A.crow + a);
-        prefetch_l2(A.cv + a);
-    }
 }
 
 template <class T, int KT>
