@@ -5,9 +5,11 @@
 // (k_flow_stage).
 //
 // What bounds it: the chain of levels.  One hop of a grid-wide kernel is a
-// store to L2 and a poll that sees it (870-1,000 cycles measured between two
-// SMs); a store into another SM's shared memory is seen after 380, one inside
-// the SM after 210, and FP64 adds 64 cycles for each dependent operation.  So
+// store to L2 and a poll that sees it (870 cycles measured between most SMs);
+// a store into the shared memory of another SM of the cluster is seen after
+// 280, one inside the SM after 160 (one lane polling; a warp that polls and
+// votes takes about 100 more), and FP64 adds 64 cycles for each dependent
+// operation.  So
 // the rows of a level are shared by the blocks of one cluster, every block
 // keeps the recent solutions its rows depend on in a ring in shared memory,
 // and a row's solution is stored into the ring of every block that needs it
@@ -32,8 +34,8 @@ namespace {
 // ------------------------------------------------------------ solution ring
 // Code of position q: bit 31, its generation q / R + 1 and its slot q mod R of
 // the shared-memory ring; a dependency too old for the ring has its row + 1 as
-// its code (bit 31 clear), no dependency 0.  A slot holds a solution together with its position's
-// code: FP32 {bits, code} in one 64-bit word; FP64 two words {low bits, code}
+// its code (bit 31 clear), no dependency 0.  A slot holds a solution together
+// with its position's code: FP32 {bits, code} in one 64-bit word; FP64 two words {low bits, code}
 // and {high bits, code}, each checked on its own, so that only the single-copy
 // atomicity of 64-bit accesses is relied on.
 constexpr uint32_t kNear = 0x80000000u;

@@ -91,8 +91,9 @@ struct Strips {
 
 // ---------------------------------------------------------------- launchers
 // Raises the dynamic shared memory that a kernel may take on the current
-// device, once per device.
-template <auto Kernel> cudaError_t allow_smem(int bytes)
+// device, once per device.  (static: a flag of external linkage would be one for
+// all builds of the library in a process, whose kernels are not the same.)
+template <auto Kernel> static cudaError_t allow_smem(int bytes)
 {
     static DeviceOnce once;  // one per kernel instantiation
     int device = -1;
