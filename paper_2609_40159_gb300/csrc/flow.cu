@@ -7,9 +7,8 @@
 // What bounds it: the chain of levels.  One hop of a grid-wide kernel is a
 // store to L2 and a poll that sees it (870 cycles measured between most SMs);
 // a store into the shared memory of another SM of the cluster is seen after
-// 280, one inside the SM after 160 (one lane polling; a warp that polls and
-// votes takes about 100 more), and FP64 adds 64 cycles for each dependent
-// operation.  So
+// 280, one inside the SM after 160 (one lane polling), and FP64 adds 64 cycles
+// for each dependent operation.  So
 // the rows of a level are shared by the blocks of one cluster, every block
 // keeps the recent solutions its rows depend on in a ring in shared memory,
 // and a row's solution is stored into the ring of every block that needs it
